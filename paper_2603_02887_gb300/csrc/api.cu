@@ -71,9 +71,16 @@ void stage_end(ngs_ctx* ctx, cudaStream_t s, int stage, cudaEvent_t start, int l
 // Host <-> device traffic of a render without the copy engines: a render would otherwise wait for its
 // view table and its pair count behind whatever bulk copies other streams have queued on the engines.
 // The view table is read by a kernel from mapped pinned memory over the host link...
-__global__ void copy_words_kernel(const uint32_t* __restrict__ src, uint32_t* __restrict__ dst, uint32_t n) {
+// (the same launch clears what the binning counts in: the tile ranges, the work list's counters, the scan's words)
+__global__ void begin_frame_kernel(const uint32_t* __restrict__ src, uint32_t* __restrict__ dst, uint32_t n,
+                                   uint2* __restrict__ ranges, uint32_t ntiles, uint32_t* __restrict__ sched,
+                                   uint64_t* total) {
   pdl_wait();
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i];
+  const uint32_t first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  for (uint32_t i = first; i < n; i += step) dst[i] = src[i];
+  for (uint32_t i = first; i < ntiles; i += step) ranges[i] = make_uint2(0, 0);
+  if (sched && first < (uint32_t)kSchedWords) sched[first] = 0;
+  if (first == 0) total[kTotalTicket] = total[kTotalBig] = 0;
 }
 
 // ... and the scalars the host reads back (the pair count and the error word, loss sums, a densified count)
@@ -224,8 +231,8 @@ static BufferPlan plan_buffers(uint64_t R, uint32_t n, uint32_t n_views, uint64_
   b.work = schedule == NGS_SCHEDULE_PERSISTENT ? sizeof(uint32_t) * (size_t)std::max<uint64_t>(ntiles, 1) : 0;
   b.sched = schedule == NGS_SCHEDULE_PERSISTENT ? sizeof(uint32_t) * kSchedWords : 0;
   b.pair_tile = b.pair_val = sizeof(uint32_t) * (size_t)std::max<uint64_t>(cap, 1);
-  b.scan_tmp = sizeof(uint64_t) * scan_tmp_words((uint32_t)R);
-  b.total = 2 * sizeof(uint64_t);
+  b.scan_tmp = sizeof(uint64_t) * std::max(scan_tmp_words((uint32_t)R), bin_bases_words(ntiles));
+  b.total = kTotalWords * sizeof(uint64_t);
   b.hist1 = sizeof(uint32_t) * radix_hist_words(std::max(n, 1u), std::max(n_views, 1u));
   b.hist2 = sizeof(uint32_t) * radix_hist_words((uint32_t)std::max<uint64_t>(cap, 1), 1);
   b.grad2d = sizeof(float4) * 3 * r1;
@@ -270,7 +277,13 @@ static size_t plan_frame_fixed(const BufferPlan& b) {
          fresh_bytes(b.offsets) + fresh_bytes(b.ranges) + fresh_bytes(b.state) + fresh_bytes(b.views) +
          fresh_bytes(b.work) + fresh_bytes(b.sched);
 }
-static size_t plan_frame_pairs(const BufferPlan& b) { return 2 * fresh_bytes(b.pair_tile) + 2 * fresh_bytes(b.pair_val); }
+static size_t pair_keys_bytes(const BufferPlan& b) { return 2 * fresh_bytes(b.pair_tile); }  // one buffer, in halves
+static size_t plan_frame_pairs(const BufferPlan& b) { return pair_keys_bytes(b) + 2 * fresh_bytes(b.pair_val); }
+
+// Which of the two ways builds the tile lists: counting (per-tile segments sorted on their own) or the global
+// radix sorts.
+constexpr uint64_t kBinMaxRecordsPerTile = 1024;
+static bool use_bins(uint64_t R, uint64_t ntiles) { return R <= kBinMaxRecordsPerTile * ntiles; }
 static size_t plan_context(const BufferPlan& b) {
   return fresh_bytes(b.scan_tmp) + fresh_bytes(b.total) + grown_size(grown_size(0, b.hist1), b.hist2);
 }
@@ -317,13 +330,21 @@ struct RenderPlan {
   uint64_t pix_total;
   float* image;
   int32_t* overdraw;
+  bool bins;  // tile lists by counting
 };
+
+// Where the counting keeps each record's tiles: the arrays that the radix sort would take its keys and order from.
+static TileMasks tile_masks(ngs_frame* f) {
+  return TileMasks{f->gkeys[0].as<uint32_t>(), f->gkeys[1].as<uint32_t>(), f->gvals[0].as<uint32_t>(),
+                   f->gvals[1].as<uint32_t>()};
+}
 
 // Phase 1: view table upload, projection, depth sort, scan of the tile counts, and the pair count (and the
 // device error word) written into the context's mapped pinned mirror. Launches only.
 static cudaError_t phase1(ngs_ctx* ctx, ngs_frame* f, const RenderPlan& pl, cudaStream_t s) {
   const RenderParams& rp = pl.rp;
   const ViewParams* views = f->views.as<ViewParams>();
+  uint32_t* sched = rp.schedule == NGS_SCHEDULE_PERSISTENT ? f->sched.as<uint32_t>() : nullptr;
   cudaEvent_t ev;
   // 1. the view table to the device; projection of every (view, Gaussian): splat records, FP32 depth keys
   //    (all-ones for splats that take no tile), tile counts
@@ -331,12 +352,23 @@ static cudaError_t phase1(ngs_ctx* ctx, ngs_frame* f, const RenderPlan& pl, cuda
   {
     static_assert(sizeof(ViewParams) % 4 == 0, "the view table is copied in 4-byte words");
     const uint32_t words = (uint32_t)(sizeof(ViewParams) * f->view_host.size() / 4);
-    launch_pdl(copy_words_kernel, std::min((words + 255) / 256, 64u), 256, 0, s, f->d_h_views, f->views.as<uint32_t>(),
-               words);
+    const uint32_t most = std::max(words, pl.ntiles / 4);
+    launch_pdl(begin_frame_kernel, std::min((most + 255) / 256, (uint32_t)ctx->num_sms), 256, 0, s, f->d_h_views,
+               f->views.as<uint32_t>(), words, f->ranges.as<uint2>(), pl.ntiles, sched,
+               ctx->total.as<uint64_t>());
   }
   launch_project(*pl.g, views, f->view_host[0].cam, rp, f->rec.as<float4>(), f->gkeys[0].as<uint32_t>(),
-                 f->tile_count.as<uint32_t>(), f->gvals[0].as<uint32_t>(), s);
+                 f->tile_count.as<uint32_t>(), f->gvals[0].as<uint32_t>(), pl.bins ? f->ranges.as<uint2>() : nullptr,
+                 tile_masks(f), s);
   stage_end(ctx, s, 0, ev, pl.n ? 2 : 1);
+  if (pl.bins) {
+    // 2. each tile's segment of the pair array, and the pair count to the host mirror
+    stage_begin(ctx, s, 2, &ev);
+    launch_tile_scan(f->ranges.as<uint2>(), pl.ntiles, ctx->scan_tmp.as<uint64_t>(), ctx->total.as<uint64_t>(),
+                     f->offsets.as<uint32_t>(), pl.R + 1, sched, ctx->d_h_total + kMirrorTotal, s);
+    stage_end(ctx, s, 2, ev, 1);
+    return cudaSuccess;
+  }
   // 2. stable sort of each view's splats by FP32 depth (ties keep Gaussian order)
   stage_begin(ctx, s, 1, &ev);
   int launches = 0;
@@ -364,43 +396,54 @@ static cudaError_t phase2(ngs_ctx* ctx, ngs_frame* f, const RenderPlan& pl, uint
   const RenderParams& rp = pl.rp;
   const ViewParams* views = f->views.as<ViewParams>();
   cudaEvent_t ev;
-  // zeroing first, so that the kernels from the emission to the composite follow one another directly
-  // (programmatic dependent launches)
-  cudaError_t e = cudaMemsetAsync(f->ranges.p, 0, sizeof(uint2) * (size_t)pl.ntiles, s);
-  if (e == cudaSuccess && rp.schedule == NGS_SCHEDULE_PERSISTENT)
-    e = cudaMemsetAsync(f->sched.p, 0, sizeof(uint32_t) * kSchedWords, s);
-  if (e != cudaSuccess) return e;
-  stage_begin(ctx, s, 2, &ev);
-  launch_emit_pairs(f->rec.as<float4>(), f->gvals[f->g_final].as<uint32_t>(), f->offsets.as<uint32_t>(), views, rp,
-                    f->ptile[0].as<uint32_t>(), f->pvals[0].as<uint32_t>(), cap, s);
-  stage_end(ctx, s, 2, ev, pl.R ? 1 : 0);
-  // 4. stable sort of the pairs by view-local tile: the (view, depth) order inside each local tile is kept,
-  //    so every (view, tile) list is contiguous and in the order of the 64-bit (tile << 32 | depth) keys
-  stage_begin(ctx, s, 3, &ev);
-  int launches = 0;
-  {
-    uint32_t* k2[2] = {f->ptile[0].as<uint32_t>(), f->ptile[1].as<uint32_t>()};
-    uint32_t* v2[2] = {f->pvals[0].as<uint32_t>(), f->pvals[1].as<uint32_t>()};
-    int max_tiles = 0;  // the pairs carry view-local tiles
-    for (const ViewParams& vp : f->view_host) max_tiles = std::max(max_tiles, vp.tiles_x * vp.tiles_y);
-    f->p_final = radix_sort_u32(k2, v2, cap, 1, np_dev, 0, tile_bits((uint32_t)max_tiles), ctx->hist.as<uint32_t>(), s,
-                                &launches);
-  }
-  stage_end(ctx, s, 3, ev, launches);
-  // 5. per-tile [start, end); for the persistent schedule, the tiles by descending pair count
-  stage_begin(ctx, s, 4, &ev);
-  launches = cap ? 1 : 0;
-  launch_tile_ranges(f->ptile[f->p_final].as<uint32_t>(), f->pvals[f->p_final].as<uint32_t>(), views, pl.n, rp.n_views,
-                     cap, np_dev, pl.ntiles, f->ranges.as<uint2>(), rp.check, s);
   const uint32_t* work = nullptr;
   uint32_t* counter = nullptr;
   if (rp.schedule == NGS_SCHEDULE_PERSISTENT) {
-    launch_tile_order(f->ranges.as<uint2>(), pl.ntiles, f->sched.as<uint32_t>(), f->work.as<uint32_t>(), s,
-                      &launches);
     work = f->work.as<uint32_t>();
     counter = f->sched.as<uint32_t>();
   }
-  stage_end(ctx, s, 4, ev, launches);
+  int launches = 0;
+  if (pl.bins) {
+    // 3. every record's keys into the segments of the tiles it covers
+    stage_begin(ctx, s, 2, &ev);
+    if (cap)
+      launch_emit_bins(f->rec.as<float4>(), f->tile_count.as<uint32_t>(), tile_masks(f), views, rp,
+                       f->ranges.as<uint2>(), ctx->scan_tmp.as<uint64_t>(), f->ptiles.as<uint64_t>(), cap, s);
+    stage_end(ctx, s, 2, ev, cap && pl.R ? 1 : 0);
+    // 4. each segment sorted by (depth, record); final ranges and work list
+    stage_begin(ctx, s, 3, &ev);
+    f->p_final = 0;
+    launch_tile_sort(f->ptiles.as<uint64_t>(), cap, ctx->scan_tmp.as<uint64_t>(), pl.ntiles, f->ranges.as<uint2>(),
+                     f->pvals[0].as<uint32_t>(), f->offsets.as<uint32_t>(), pl.R + 1, ctx->total.as<uint64_t>(), counter,
+                     f->work.as<uint32_t>(), ctx->num_sms, s);
+    stage_end(ctx, s, 3, ev, 1);
+  } else {
+    stage_begin(ctx, s, 2, &ev);
+    launch_emit_pairs(f->rec.as<float4>(), f->gvals[f->g_final].as<uint32_t>(), f->offsets.as<uint32_t>(), views, rp,
+                      f->ptile(0), f->pvals[0].as<uint32_t>(), cap, s);
+    stage_end(ctx, s, 2, ev, pl.R ? 1 : 0);
+    // 4. stable sort of the pairs by view-local tile: the (view, depth) order inside each local tile is kept,
+    //    so every (view, tile) list is contiguous and in the order of the 64-bit (tile << 32 | depth) keys
+    stage_begin(ctx, s, 3, &ev);
+    {
+      uint32_t* k2[2] = {f->ptile(0), f->ptile(1)};
+      uint32_t* v2[2] = {f->pvals[0].as<uint32_t>(), f->pvals[1].as<uint32_t>()};
+      int max_tiles = 0;  // the pairs carry view-local tiles
+      for (const ViewParams& vp : f->view_host) max_tiles = std::max(max_tiles, vp.tiles_x * vp.tiles_y);
+      f->p_final = radix_sort_u32(k2, v2, cap, 1, np_dev, 0, tile_bits((uint32_t)max_tiles), ctx->hist.as<uint32_t>(),
+                                  s, &launches);
+    }
+    stage_end(ctx, s, 3, ev, launches);
+    // 5. per-tile [start, end); for the persistent schedule, the tiles by descending pair count
+    stage_begin(ctx, s, 4, &ev);
+    launches = cap ? 1 : 0;
+    launch_tile_ranges(f->ptile(f->p_final), f->pvals[f->p_final].as<uint32_t>(), views, pl.n, rp.n_views, cap, np_dev,
+                       pl.ntiles, f->ranges.as<uint2>(), rp.check, s);
+    if (counter)
+      launch_tile_order(f->ranges.as<uint2>(), pl.ntiles, f->sched.as<uint32_t>(), f->work.as<uint32_t>(), s,
+                        &launches);
+    stage_end(ctx, s, 4, ev, launches);
+  }
   // 6. composite every tile of every view
   stage_begin(ctx, s, 5, &ev);
   launch_composite_forward(f->rec.as<float4>(), f->pvals[f->p_final].as<uint32_t>(), f->ranges.as<uint2>(), rp, views,
@@ -577,6 +620,7 @@ int ngs::render_views_out(ngs_ctx* ctx, ngs_frame* f, const ngs_gaussians* g, co
   pl.R = rp.n_records;
   pl.ntiles = rp.n_tiles;
   pl.pix_total = pix_total;
+  pl.bins = use_bins(records64, tiles_total);
   pl.image = images[0];
   pl.overdraw = overdraws ? overdraws[0] : nullptr;
   const uint32_t R = pl.R;
@@ -597,7 +641,7 @@ int ngs::render_views_out(ngs_ctx* ctx, ngs_frame* f, const ngs_gaussians* g, co
   NGS_TRY(ensure(ctx, ctx->scan_tmp, bp.scan_tmp));
   if (!ctx->total.p) {
     NGS_TRY(ensure(ctx, ctx->total, bp.total));
-    const cudaError_t ze = cudaMemsetAsync(ctx->total.p, 0, 2 * sizeof(uint64_t), s);
+    const cudaError_t ze = cudaMemsetAsync(ctx->total.p, 0, kTotalWords * sizeof(uint64_t), s);
     if (ze != cudaSuccess) {
       free_buf(ctx->total);  // zeroed on the next render's first use again
       return fail(ctx, NGS_ERR_CUDA, std::string("clearing the pair count: ") + cudaGetErrorString(ze));
@@ -627,6 +671,7 @@ int ngs::render_views_out(ngs_ctx* ctx, ngs_frame* f, const ngs_gaussians* g, co
   for (const DevBuf* b : {&f->rec, &f->tile_count, &f->gkeys[0], &f->gkeys[1], &f->gvals[0], &f->gvals[1], &f->offsets,
                           &f->views, &ctx->hist, &ctx->scan_tmp, &ctx->total})
     k1.add(b->p);
+  for (const DevBuf* b : {&f->ranges, &f->sched}) k1.add(b->p);
   k1.add(f->h_views);
   k1.add(ctx->h_total);
   // asynchronous: no host synchronisation; phase 2 is sized by the frame's capacity (set by earlier renders)
@@ -666,10 +711,8 @@ int ngs::render_views_out(ngs_ctx* ctx, ngs_frame* f, const ngs_gaussians* g, co
     }
   }
   const BufferPlan bp2 = plan_buffers(R, pl.n, (uint32_t)n_views, pl.ntiles, pix_total, rp.schedule, cap);
-  for (int k = 0; k < 2; ++k) {
-    NGS_TRY(ensure(ctx, f->ptile[k], bp2.pair_tile));
-    NGS_TRY(ensure(ctx, f->pvals[k], bp2.pair_val));
-  }
+  NGS_TRY(ensure(ctx, f->ptiles, pair_keys_bytes(bp2)));
+  for (int k = 0; k < 2; ++k) NGS_TRY(ensure(ctx, f->pvals[k], bp2.pair_val));
   NGS_TRY(ensure(ctx, ctx->hist, bp2.hist2));
   KeyBuf k2;
   k2.add(rp);
@@ -684,8 +727,10 @@ int ngs::render_views_out(ngs_ctx* ctx, ngs_frame* f, const ngs_gaussians* g, co
     k2.add(vp.tiles_x);
     k2.add(vp.tiles_y);
   }
-  for (const DevBuf* b : {&f->rec, &f->gvals[0], &f->gvals[1], &f->offsets, &f->views, &f->ptile[0], &f->ptile[1],
-                          &f->pvals[0], &f->pvals[1], &ctx->hist, &f->ranges, &f->work, &f->sched, &f->state})
+  for (const DevBuf* b : {&f->rec, &f->gkeys[0], &f->gkeys[1], &f->gvals[0], &f->gvals[1], &f->offsets, &f->views,
+                          &f->ptiles, &f->tile_count, &ctx->total,
+                          &f->pvals[0], &f->pvals[1], &ctx->hist, &ctx->scan_tmp, &f->ranges, &f->work, &f->sched,
+                          &f->state})
     k2.add(b->p);
   if (async) k2.add(f->d_status);
   NGS_TRY(run_phase(ctx, f, 1, k2, s, [&](cudaStream_t st) { return phase2(ctx, f, pl, cap, np_dev, async, st); }));
@@ -776,7 +821,7 @@ NGS_API void ngs_frame_destroy(ngs_frame* f) {
   if (!f) return;
   cudaDeviceSynchronize();
   DevBuf* bufs[] = {&f->rec,     &f->tile_count, &f->gkeys[0], &f->gkeys[1], &f->gvals[0], &f->gvals[1],
-                    &f->offsets, &f->ptile[0],   &f->ptile[1], &f->pvals[0], &f->pvals[1], &f->ranges,
+                    &f->offsets, &f->ptiles,     &f->pvals[0], &f->pvals[1], &f->ranges,
                     &f->state,   &f->views,      &f->keys64,   &f->work,     &f->sched};
   for (DevBuf* b : bufs) free_buf(*b);
   if (f->h_views) cudaFreeHost(f->h_views);
@@ -910,9 +955,8 @@ NGS_API int ngs_frame_view_get(const ngs_frame* fc, ngs_frame_view* out) {
   if (ensure(f->ctx, f->keys64, sizeof(uint64_t) * (size_t)std::max(np, 1u)) != NGS_OK) return NGS_ERR_OUT_OF_MEMORY;
   cudaError_t e = cudaDeviceSynchronize();
   if (e == cudaSuccess) {
-    launch_compose_keys(f->ptile[f->p_final].as<uint32_t>(), f->pvals[f->p_final].as<uint32_t>(), f->rec.as<float4>(),
-                        f->views.as<ViewParams>(), (uint32_t)f->n, (uint32_t)f->n_views, np, f->keys64.as<uint64_t>(),
-                        nullptr);
+    launch_compose_keys(f->ranges.as<uint2>(), f->rp.n_tiles, f->pvals[f->p_final].as<uint32_t>(), f->rec.as<float4>(),
+                        f->keys64.as<uint64_t>(), nullptr);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
@@ -1020,7 +1064,7 @@ NGS_API int ngs_memory_usage(const ngs_ctx* ctx, const ngs_frame* f, size_t* ctx
     *frame_bytes = 0;
     if (f)
       for (const DevBuf* b : {&f->rec, &f->tile_count, &f->gkeys[0], &f->gkeys[1], &f->gvals[0], &f->gvals[1],
-                              &f->offsets, &f->ptile[0], &f->ptile[1], &f->pvals[0], &f->pvals[1], &f->ranges,
+                              &f->offsets, &f->ptiles, &f->pvals[0], &f->pvals[1], &f->ranges,
                               &f->state, &f->views, &f->keys64, &f->work, &f->sched})
         *frame_bytes += b->p ? b->cap : 0;
   }

@@ -280,7 +280,8 @@ struct ngs_frame {
   cudaEvent_t views_uploaded = nullptr;    // recorded after the last upload from h_views
   ngs::DevBuf views;                       // device view table
   ngs::DevBuf rec, tile_count, gkeys[2], gvals[2], offsets;
-  ngs::DevBuf ptile[2], pvals[2], ranges, state;
+  ngs::DevBuf ptiles;  // 8 B per pair: the pairs' keys (depth, record), or the radix sort's two tile arrays
+  ngs::DevBuf pvals[2], ranges, state;
   ngs::DevBuf keys64;  // 64-bit keys, materialised only for ngs_frame_view_get
   ngs::DevBuf work;    // persistent schedule: tiles by descending pair count
   ngs::DevBuf sched;   // persistent schedule: kSchedWords counters (see launch_tile_order)
@@ -296,7 +297,8 @@ struct ngs_frame {
   uint64_t* d_status = nullptr;
   cudaEvent_t done = nullptr;
   int g_final = 0;  // which gvals[] holds the depth-sorted Gaussian order
-  int p_final = 0;  // which ptile[]/pvals[] hold the sorted pairs
+  int p_final = 0;  // which pvals[] holds the sorted pairs' record indices
+  uint32_t* ptile(int k) const { return ptiles.as<uint32_t>() + (k ? ptiles.cap / 8 : 0); }  // radix sort
 };
 
 namespace ngs {
@@ -335,11 +337,20 @@ void stage_begin(ngs_ctx* ctx, cudaStream_t s, int stage, cudaEvent_t* out);
 void stage_end(ngs_ctx* ctx, cudaStream_t s, int stage, cudaEvent_t start, int launches);
 
 // kernels' host launchers
+// The tiles a record covers, as the projection found them: bit 8 (ty - y0) + (tx - x0) of the mask for a bounding box of
+// at most 8 x 8 tiles at (x0, y0) = (box & 0xFFFF, box >> 16); kLargeBox for a larger one. One array each, by record.
+struct TileMasks {
+  uint32_t *lo, *hi, *box, *zbits;  // zbits: the FP32 depth's bits
+};
+constexpr uint32_t kLargeBox = 0xFFFFFFFFu;
 // For every view v and Gaussian i, record r = v n + i: splat record, depth key (0xFFFFFFFF for splats
 // without tiles), tile count and order[r] = r.
-// cam0: the camera of view 0 (used when rp.n_views == 1).
+// cam0: the camera of view 0 (used when rp.n_views == 1). With `bins` (the zeroed tile ranges), every covered
+// tile's count is added up in bins[].y and the records' tiles are kept in `masks`; depth_key and order are then not
+// written.
 void launch_project(const ngs_gaussians& g, const ViewParams* views, const CamParams& cam0, const RenderParams& rp,
-                    float4* rec, uint32_t* depth_key, uint32_t* tile_count, uint32_t* order, cudaStream_t s);
+                    float4* rec, uint32_t* depth_key, uint32_t* tile_count, uint32_t* order, uint2* bins,
+                    const TileMasks& masks, cudaStream_t s);
 // Gradients w.r.t. the Gaussian parameters, summed over the views.
 // cam0: the camera of view 0 (the only one when rp.n_views == 1).
 void launch_project_backward(const ngs_gaussians& g, const ViewParams* views, const CamParams& cam0,
@@ -364,9 +375,28 @@ size_t scan_tmp_words(uint32_t n);
 // Pairs at slots >= cap are not written (an asynchronous render whose count exceeds its capacity).
 void launch_emit_pairs(const float4* rec, const uint32_t* order, const uint32_t* offsets, const ViewParams* views,
                        const RenderParams& rp, uint32_t* tiles, uint32_t* vals, uint32_t cap, cudaStream_t s);
-// keys[i] = global tile of pair i << 32 | bits(depth of record vals[i]) (diagnostics).
-void launch_compose_keys(const uint32_t* tiles, const uint32_t* vals, const float4* rec, const ViewParams* views,
-                         uint32_t n_per_view, uint32_t n_views, uint32_t npairs, uint64_t* keys, cudaStream_t s);
+// keys[i] = tile << 32 | bits(depth of record ids[i]) for every pair of every tile's list (diagnostics).
+void launch_compose_keys(const uint2* ranges, uint32_t ntiles, const uint32_t* ids, const float4* rec, uint64_t* keys,
+                         cudaStream_t s);
+// Per-tile lists by counting (sort.cu). The scan turns the counts in ranges[].y into each tile's first pair
+// relative to its block of kBinBlock tiles, `bases` into the blocks' first pairs, and writes the pair count to
+// total[0] and (with the error word total[1]) to the host mirror; total[kTotalTicket] is zeroed by the caller.
+// Tiles with long lists are listed in `big`.
+constexpr int kBinBlock = 1024;
+constexpr int kTotalTicket = 2, kTotalBig = 3, kTotalWords = 4;
+size_t bin_bases_words(uint64_t ntiles);
+void launch_tile_scan(uint2* ranges, uint32_t ntiles, uint64_t* bases, uint64_t* total, uint32_t* big, uint32_t big_cap,
+                      uint32_t* sched, uint64_t* mirror, cudaStream_t s);
+// One (depth bits << 32 | record) key per covered tile into the tile's segment, in any order; slots past cap
+// are not written.
+void launch_emit_bins(const float4* rec, const uint32_t* tile_count, const TileMasks& masks, const ViewParams* views,
+                      const RenderParams& rp, uint2* ranges, const uint64_t* bases, uint64_t* keys, uint32_t cap,
+                      cudaStream_t s);
+// Sorts each tile's segment of keys; the record indices go to out, the final [start, end) to ranges, and (with
+// sched) the tiles to the work list of the persistent schedule. The segments of keys are scratch afterwards.
+void launch_tile_sort(uint64_t* keys, uint32_t cap, const uint64_t* bases, uint32_t ntiles, uint2* ranges, uint32_t* out,
+                      const uint32_t* big, uint32_t big_cap, const uint64_t* total, uint32_t* sched, uint32_t* work,
+                      int num_sms, cudaStream_t s);
 // [start, end) of every global tile's pairs into `ranges`, which the caller has zeroed (zero-length ranges
 // stay (0, 0)); npairs_cap items are covered by the grid, of which the first *npairs_dev are valid if
 // npairs_dev is not null. A pair naming a record or tile out of range is skipped and reported in *check.

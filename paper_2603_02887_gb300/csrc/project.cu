@@ -343,19 +343,33 @@ __device__ __forceinline__ bool tile_rect(float u, float v, float rx, float ry, 
   return true;
 }
 
-// Tiles covered over tile rows [y0, y1] (columns clipped to [x0, x1]).
+// Adds one splat to the counts of tiles [t0, t1] of tile row ty (`bins`: the view's tiles).
+__device__ __forceinline__ void add_to_bins(uint2* bins, const RenderParams& rp, int ty, int t0, int t1) {
+  uint2* b = bins + (int64_t)ty * rp.tiles_x;
+  for (int tx = t0; tx <= t1; ++tx) atomicAdd(&b[tx].y, 1u);
+}
+
+// Tiles covered over tile rows [y0, y1] (columns clipped to [x0, x1]), added to the tiles' counts if `bins`; mask:
+// their bits in the box's 8 x 8 tiles (columns past the eighth are left out: the caller discards it then).
 __device__ __forceinline__ uint32_t count_rows(const SplatBin& b, const RenderParams& rp, int x0, int x1, int y0,
-                                               int y1) {
+                                               int y1, uint2* bins, uint2& mask) {
   uint32_t c = 0;
   for (int ty = y0; ty <= y1; ++ty) {
     int t0, t1;
-    if (row_span(b, rp, ty, x0, x1, t0, t1)) c += (uint32_t)(t1 - t0 + 1);
+    if (!row_span(b, rp, ty, x0, x1, t0, t1)) continue;
+    c += (uint32_t)(t1 - t0 + 1);
+    if (bins) {
+      add_to_bins(bins, rp, ty, t0, t1);
+      const uint32_t bits = (((2u << min(t1 - x0, 7)) - (1u << min(t0 - x0, 7))) & 0xFFu) << (8 * ((ty - y0) & 3));
+      if (ty - y0 < 4) mask.x |= bits;
+      else mask.y |= bits;
+    }
   }
   return c;
 }
 
 // A splat spanning more tile rows than this has them counted by its whole warp, one row per lane.
-constexpr int kCoopRows = 8;
+constexpr int kCoopRows = 8;  // (the rows of a tile mask)
 
 // Block b works on view b % n_views and Gaussians [256 (b / n_views), +256): the views of one block of
 // Gaussians run side by side, so their parameters are read from HBM once and from L2 afterwards.
@@ -364,7 +378,8 @@ constexpr int kCoopRows = 8;
 template <int DEG, bool VEC>
 __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const ViewParams* __restrict__ views,
                                                       CamParams cam0, RenderParams rp, float4* rec,
-                                                      uint32_t* depth_key, uint32_t* tile_count, uint32_t* order) {
+                                                      uint32_t* depth_key, uint32_t* tile_count, uint32_t* order,
+                                                      uint2* bins, TileMasks masks) {
   pdl_wait();
   const uint32_t view = blockIdx.x % rp.n_views;
   const int i = (blockIdx.x / rp.n_views) * blockDim.x + threadIdx.x;
@@ -372,6 +387,7 @@ __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const 
   if (rp.n_views != 1) {  // the block's view (one per block)
     rp.tiles_x = views[view].tiles_x;
     rp.tiles_y = views[view].tiles_y;
+    if (bins) bins += views[view].tile_base;
   }
   const int64_t r = (int64_t)view * g.n + i;  // record index
   if (i < g.n) {
@@ -391,6 +407,7 @@ __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const 
   uint32_t count = 0;
   bool tall = false;
   int x0 = 0, x1 = -1, y0 = 0, y1 = -1;
+  uint2 mask = make_uint2(0, 0);
   SplatBin b = {};
   float z = 0.f;
   if (i < g.n) {
@@ -418,14 +435,14 @@ __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const 
         if (tile_rect(r0.x, r0.y, r2.z, r2.w, rp, x0, x1, y0, y1)) {
           b = splat_bin(r0, r1, rp.log2_alpha_min);
           tall = y1 - y0 >= kCoopRows;
-          if (!tall) count = count_rows(b, rp, x0, x1, y0, y1);
+          if (!tall) count = count_rows(b, rp, x0, x1, y0, y1, bins, mask);
         }
       }
     }
     rec[3 * r] = r0;
     rec[3 * r + 1] = r1;
     rec[3 * r + 2] = r2;
-    order[r] = (uint32_t)r;
+    if (!bins) order[r] = (uint32_t)r;
   }
   // tall splats, one after another: lane l counts tile rows y0 + l, y0 + l + 32, ... (the same row spans)
   for (uint32_t pending = __ballot_sync(0xFFFFFFFFu, tall); pending != 0u; pending &= pending - 1u) {
@@ -444,13 +461,22 @@ __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const 
     uint32_t c = 0;
     for (int ty = cy0 + lane; ty <= cy1; ty += 32) {
       int t0, t1;
-      if (row_span(cb, rp, ty, cx0, cx1, t0, t1)) c += (uint32_t)(t1 - t0 + 1);
+      if (!row_span(cb, rp, ty, cx0, cx1, t0, t1)) continue;
+      c += (uint32_t)(t1 - t0 + 1);
+      if (bins) add_to_bins(bins, rp, ty, t0, t1);
     }
     c = __reduce_add_sync(0xFFFFFFFFu, c);
     if (lane == src) count = c;
   }
   if (i < g.n) {
-    depth_key[r] = count ? __float_as_uint(z) : 0xFFFFFFFFu;
+    if (bins) {
+      masks.lo[r] = mask.x;
+      masks.hi[r] = mask.y;
+      masks.box[r] = tall || x1 - x0 >= 8 ? kLargeBox : ((uint32_t)y0 << 16 | (uint32_t)x0);
+      masks.zbits[r] = __float_as_uint(z);
+    } else {
+      depth_key[r] = count ? __float_as_uint(z) : 0xFFFFFFFFu;
+    }
     tile_count[r] = count;
   }
 }
@@ -539,6 +565,136 @@ __global__ void __launch_bounds__(256) emit_pairs_kernel(const float4* rec, cons
         vals[o] = cid;
       }
       coff += __shfl_sync(0xFFFFFFFFu, incl, 31);
+    }
+  }
+}
+
+// Writes `key` at the next free slots of tiles [t0, t1] of one tile row (`tiles`: index of the row's tile 0).
+// Four slots are taken before the first is written to, so that the atomics' round trips overlap.
+__device__ __forceinline__ void emit_row(unsigned long long key, uint32_t tiles, int t0, int t1,
+                                         uint2* __restrict__ ranges, const uint64_t* __restrict__ bases,
+                                         unsigned long long* __restrict__ keys, uint32_t cap) {
+  for (int tx = t0; tx <= t1; tx += 4) {
+    uint64_t slot[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t t = tiles + (uint32_t)(tx + k);
+      if (tx + k <= t1) slot[k] = bases[t / kBinBlock] + atomicAdd(&ranges[t].y, 1u);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (tx + k <= t1 && slot[k] < cap) keys[slot[k]] = key;
+  }
+}
+
+// A warp takes 32 records, in record order: the tiles of their masks are listed in shared memory (a record of many
+// tiles by the whole warp, the others by their own lanes), and the warp then takes the listed pairs 256 at a time,
+// whatever record they belong to, so that every lane has a pair and eight slots' atomics are on their way at once. Records with larger bounding boxes follow one
+// by one, one tile row per lane (the row spans that the projection counted).
+constexpr int kEmitList = 1024;  // 16 masks of at most 64 tiles
+constexpr int kEmitWarps = 4;
+constexpr uint32_t kEmitOwn = 6;  // a record of up to this many tiles is listed by its own lane
+__global__ void __launch_bounds__(32 * kEmitWarps) emit_bins_kernel(const float4* __restrict__ rec,
+                                                        const uint32_t* __restrict__ tile_count, TileMasks masks,
+                                                        const ViewParams* __restrict__ views, RenderParams rp,
+                                                        uint2* __restrict__ ranges, const uint64_t* __restrict__ bases,
+                                                        unsigned long long* __restrict__ keys, uint32_t cap) {
+  pdl_wait();
+  __shared__ uint32_t s_pairs[kEmitWarps][kEmitList];
+  const uint32_t full = 0xFFFFFFFFu;
+  const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t lane = threadIdx.x & 31, first_id = id - lane;
+  uint32_t* const list = s_pairs[threadIdx.x >> 5];
+  uint32_t count = 0, box = 0, zbits = 0, tile_base = 0;
+  unsigned long long mask = 0;
+  int tiles_x = rp.tiles_x;
+  if (id < rp.n_records) {
+    count = tile_count[id];
+    mask = (unsigned long long)masks.hi[id] << 32 | masks.lo[id];
+    box = masks.box[id];
+    zbits = masks.zbits[id];
+    if (rp.n_views != 1) {
+      const ViewParams& v = views[id / rp.n_gaussians];
+      tiles_x = v.tiles_x;
+      tile_base = v.tile_base;
+    }
+  }
+  const bool large = count != 0 && box == kLargeBox;
+  if (large) mask = 0;
+  const uint32_t mine = (uint32_t)__popcll(mask);
+  uint32_t off = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(full, off, o);
+    if (lane >= (uint32_t)o) off += y;
+  }
+  const uint32_t total = __shfl_sync(full, off, 31);
+  off -= mine;
+  const uint32_t corner = (box >> 16) * (uint32_t)tiles_x + (box & 0xFFFFu);
+  // all 32 records at once, or, where the list could not hold them, 16 and then 16
+  const uint32_t half = __shfl_sync(full, off, 16);
+  for (int part = 0; part < (total > (uint32_t)kEmitList ? 2 : 1); ++part) {
+    const bool split = total > (uint32_t)kEmitList;
+    const bool turn = !split || (lane >> 4) == (uint32_t)part;
+    const uint32_t m = !split ? total : (part == 0 ? half : total - half);
+    uint32_t at = off - (part == 0 ? 0u : half);
+    for (uint32_t pending = __ballot_sync(full, turn && mine > kEmitOwn); pending != 0u; pending &= pending - 1u) {
+      const int src = __ffs(pending) - 1;
+      const uint32_t lo = __shfl_sync(full, (uint32_t)mask, src), hi = __shfl_sync(full, (uint32_t)(mask >> 32), src);
+      const uint32_t o = __shfl_sync(full, at, src), pos = __shfl_sync(full, corner, src);
+      const uint32_t tx = __shfl_sync(full, (uint32_t)tiles_x, src);
+      const uint32_t t = pos + (lane >> 3) * tx + (lane & 7), below = (1u << lane) - 1u;  // < 2^22 tiles a view
+      if (lo >> lane & 1u) list[o + __popc(lo & below)] = t << 5 | (uint32_t)src;
+      if (hi >> lane & 1u) list[o + __popc(lo) + __popc(hi & below)] = (t + 4 * tx) << 5 | (uint32_t)src;
+    }
+    if (turn && mine <= kEmitOwn) {
+      for (; mask != 0; mask &= mask - 1) {
+        const uint32_t bit = (uint32_t)__ffsll((long long)mask) - 1;
+        list[at++] = (corner + (bit >> 3) * (uint32_t)tiles_x + (bit & 7)) << 5 | lane;
+      }
+    }
+    __syncwarp();
+    constexpr int kFlight = 8;
+    for (uint32_t i0 = 0; i0 < m; i0 += 32 * kFlight) {
+      uint32_t src[kFlight], slot[kFlight];
+#pragma unroll
+      for (int k = 0; k < kFlight; ++k) {
+        const uint32_t i = i0 + 32 * k + lane;
+        const uint32_t e = i < m ? list[i] : 0u;
+        src[k] = e & 31;
+        const uint32_t t = (e >> 5) + (rp.n_views != 1 ? __shfl_sync(full, tile_base, src[k]) : 0u);
+        slot[k] = 0xFFFFFFFFu;
+        if (i < m) {
+          const uint64_t p = bases[t / kBinBlock] + atomicAdd(&ranges[t].y, 1u);
+          if (p < cap) slot[k] = (uint32_t)p;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < kFlight; ++k) {
+        const unsigned long long key = (unsigned long long)__shfl_sync(full, zbits, src[k]) << 32 | (first_id + src[k]);
+        if (slot[k] != 0xFFFFFFFFu) keys[slot[k]] = key;
+      }
+    }
+    __syncwarp();
+  }
+  for (uint32_t pending = __ballot_sync(full, large); pending != 0u; pending &= pending - 1u) {
+    const int src = __ffs(pending) - 1;
+    const uint32_t cid = first_id + src, cbase = __shfl_sync(full, tile_base, src);
+    const unsigned long long key = (unsigned long long)__shfl_sync(full, zbits, src) << 32 | cid;
+    RenderParams rv = rp;
+    if (rp.n_views != 1) {
+      const ViewParams& v = views[cid / rp.n_gaussians];
+      rv.tiles_x = v.tiles_x;
+      rv.tiles_y = v.tiles_y;
+    }
+    const float4 r0 = rec[3 * (int64_t)cid], r1 = rec[3 * (int64_t)cid + 1], r2 = rec[3 * (int64_t)cid + 2];
+    int x0, x1, y0, y1;
+    if (!tile_rect(r0.x, r0.y, r2.z, r2.w, rv, x0, x1, y0, y1)) continue;  // (never: it was counted)
+    const SplatBin b = splat_bin(r0, r1, rp.log2_alpha_min);
+    for (int ty = y0 + (int)lane; ty <= y1; ty += 32) {
+      int t0, t1;
+      if (row_span(b, rp, ty, x0, x1, t0, t1))
+        emit_row(key, cbase + (uint32_t)(ty * rv.tiles_x), t0, t1, ranges, bases, keys, cap);
     }
   }
 }
@@ -821,12 +977,14 @@ __global__ void __launch_bounds__(128, MULTI ? 1 : 4) project_backward_kernel(ng
 }  // namespace
 
 void launch_project(const ngs_gaussians& g, const ViewParams* views, const CamParams& cam0, const RenderParams& rp,
-                    float4* rec, uint32_t* depth_key, uint32_t* tile_count, uint32_t* order, cudaStream_t s) {
+                    float4* rec, uint32_t* depth_key, uint32_t* tile_count, uint32_t* order, uint2* bins,
+                    const TileMasks& masks, cudaStream_t s) {
   if (g.n == 0) return;
   unsigned blocks = (unsigned)((g.n + 255) / 256) * rp.n_views;
   bool vec = ((uintptr_t)g.sh & 15) == 0;
 #define NGS_PROJECT(D, V) \
-  launch_pdl(project_kernel<D, V>, blocks, 256, 0, s, g, views, cam0, rp, rec, depth_key, tile_count, order)
+  launch_pdl(project_kernel<D, V>, blocks, 256, 0, s, g, views, cam0, rp, rec, depth_key, tile_count, order, bins, \
+             masks)
   switch (rp.sh_degree) {
     case 0: NGS_PROJECT(0, false); break;
     case 1:
@@ -847,6 +1005,14 @@ void launch_emit_pairs(const float4* rec, const uint32_t* order, const uint32_t*
   if (rp.n_records == 0) return;
   launch_pdl(emit_pairs_kernel, (rp.n_records + 255) / 256, 256, 0, s, rec, order, offsets, views, rp, tiles, vals,
              cap);
+}
+
+void launch_emit_bins(const float4* rec, const uint32_t* tile_count, const TileMasks& masks, const ViewParams* views,
+                      const RenderParams& rp, uint2* ranges, const uint64_t* bases, uint64_t* keys, uint32_t cap,
+                      cudaStream_t s) {
+  if (rp.n_records == 0) return;
+  launch_pdl(emit_bins_kernel, (rp.n_records + 32 * kEmitWarps - 1) / (32 * kEmitWarps), 32 * kEmitWarps, 0, s, rec, tile_count, masks, views, rp,
+             ranges, bases, reinterpret_cast<unsigned long long*>(keys), cap);
 }
 
 template <int DEG, bool VEC>

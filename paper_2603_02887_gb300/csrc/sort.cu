@@ -13,6 +13,8 @@
 // orders equal depths by Gaussian index (the pairs are emitted in index order within one depth).
 // A count known only on the device (the number of pairs, inside a captured graph) is read by every
 // kernel: blocks past it contribute empty histograms and move nothing.
+#include <algorithm>
+
 #include "ngs_internal.cuh"
 
 namespace ngs {
@@ -309,13 +311,6 @@ __global__ void __launch_bounds__(kScanThreads) scan_final_kernel(const uint32_t
   }
 }
 
-// Global tile of pair i: the view's first tile plus the view-local tile it was sorted by.
-__device__ __forceinline__ uint32_t global_tile(const uint32_t* __restrict__ tiles, const uint32_t* __restrict__ vals,
-                                                const ViewParams* __restrict__ views, uint32_t n_per_view,
-                                                uint32_t n_views, uint32_t i) {
-  return n_views == 1 ? tiles[i] : __ldg(&views[vals[i] / n_per_view].tile_base) + tiles[i];
-}
-
 __global__ void tile_ranges_kernel(const uint32_t* __restrict__ tiles, const uint32_t* __restrict__ vals,
                                    const ViewParams* __restrict__ views, uint32_t n_per_view, uint32_t n_views,
                                    uint32_t npairs_cap, const uint32_t* __restrict__ npairs_dev, uint32_t ntiles,
@@ -355,15 +350,16 @@ __global__ void tile_ranges_kernel(const uint32_t* __restrict__ tiles, const uin
   if (last) ranges[t].y = i + 1;
 }
 
-__global__ void compose_keys_kernel(const uint32_t* __restrict__ tiles, const uint32_t* __restrict__ vals,
-                                    const float4* __restrict__ rec, const ViewParams* __restrict__ views,
-                                    uint32_t n_per_view, uint32_t n_views, uint32_t npairs,
-                                    uint64_t* __restrict__ keys) {
-  uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= npairs) return;
-  const float z = rec[3 * (size_t)vals[i] + 2].y;
-  const uint32_t t = global_tile(tiles, vals, views, n_per_view, n_views, i);
-  keys[i] = ((uint64_t)t << 32) | (uint64_t)__float_as_uint(z);
+// One warp per tile: the 64-bit keys of its list (diagnostics).
+__global__ void __launch_bounds__(256) compose_keys_kernel(const uint2* __restrict__ ranges, uint32_t ntiles,
+                                                           const uint32_t* __restrict__ ids,
+                                                           const float4* __restrict__ rec,
+                                                           uint64_t* __restrict__ keys) {
+  const uint32_t t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (t >= ntiles) return;
+  const uint2 r = ranges[t];
+  for (uint32_t i = r.x + (threadIdx.x & 31); i < r.y; i += 32)
+    keys[i] = ((uint64_t)t << 32) | (uint64_t)__float_as_uint(rec[3 * (size_t)ids[i] + 2].y);
 }
 
 // ---- tile work order for the persistent composite: descending pair count ---------------------------
@@ -407,6 +403,438 @@ __global__ void __launch_bounds__(256) tile_bucket_scatter_kernel(const uint2* _
   if (b < (uint32_t)kCostBuckets && lane == leader) base = atomicAdd(&cursors[b], (uint32_t)__popc(peers));
   base = __shfl_sync(0xFFFFFFFFu, base, leader);
   if (b < (uint32_t)kCostBuckets) work[s_start[b] + base + __popc(peers & ((1u << lane) - 1u))] = t;
+}
+
+// ---- per-tile lists by counting ------------------------------------------------------------------------
+//
+// The lists of all tiles without a global sort: the projection counts every tile's splats, a scan of the
+// counts gives each tile its segment of the pair array, the emission drops each (depth, record) pair at the
+// next free slot of its tile's segment, in any order, and tile_sort_kernel sorts every segment by
+// (depth, record index). That is the order the two stable radix sorts give, with each pair written and read
+// once (8 B) and 4 B written, instead of 3 radix passes' worth of 16 B, and 3 kernels instead of about 20.
+
+constexpr int kBinThreads = 256;
+static_assert(kBinBlock == 4 * kBinThreads, "four tiles per thread");
+static_assert(kCostBuckets == 33, "a warp and one more");
+constexpr int kSortThreads = 256;
+constexpr int kWarpList = 256;     // longest list sorted by one warp
+constexpr int kWarpBuckets = 256;  // its buckets
+constexpr int kCtaList = kWarpList * (kSortThreads / 32);  // keys a CTA holds in shared memory
+constexpr int kCtaBuckets = kWarpBuckets * (kSortThreads / 32);
+constexpr uint32_t kHeavy = 48;  // a bucket with more keys is sorted by the network, not by counting
+
+// ranges[t].y holds tile t's count; afterwards ranges[t] = (o, o) with o the number of pairs in the tiles
+// before t of its block of kBinBlock tiles. `bases` receives the blocks' first pairs, *total the pair count:
+// the block that finishes last scans the blocks' sums, so that no block waits on another. Tiles whose lists are
+// too long for one warp are listed in `big` (as far as its big_cap entries go; total[kTotalBig] counts them all).
+// With `sched`, the work list's first entry of each cost bucket is left in the bucket's cursor. The count and the
+// device error word are published in the host mirror.
+__global__ void __launch_bounds__(kBinThreads) tile_scan_kernel(uint2* __restrict__ ranges, uint32_t ntiles,
+                                                                uint64_t* bases, uint64_t* total,
+                                                                uint32_t* __restrict__ big, uint32_t big_cap,
+                                                                uint32_t* sched, uint64_t* mirror) {
+  pdl_wait();
+  __shared__ uint32_t s_warp[kBinThreads / 32];
+  __shared__ uint64_t s_warp64[kBinThreads / 32];
+  __shared__ uint32_t s_cost[kCostBuckets];
+  __shared__ bool s_last;
+  const int tid = threadIdx.x;
+  if (sched) {
+    if (tid < kCostBuckets) s_cost[tid] = 0;
+    __syncthreads();
+  }
+  const uint32_t t0 = blockIdx.x * (uint32_t)kBinBlock + 4 * tid;
+  uint32_t c[4], sum = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    c[k] = t0 + k < ntiles ? ranges[t0 + k].y : 0u;
+    if (sched && t0 + k < ntiles) atomicAdd(&s_cost[cost_bucket(make_uint2(0, c[k]))], 1u);
+    sum += c[k];
+    if (c[k] > (uint32_t)kWarpList) {
+      const uint32_t at = atomicAdd(reinterpret_cast<uint32_t*>(total + kTotalBig), 1u);
+      if (at < big_cap) big[at] = t0 + k;
+    }
+  }
+  uint32_t agg;
+  uint32_t run = block_exclusive_sum<kBinThreads>(sum, s_warp, &agg);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (t0 + k < ntiles) ranges[t0 + k] = make_uint2(run, run);
+    run += c[k];
+  }
+  if (sched && tid < kCostBuckets && s_cost[tid]) {
+    atomicAdd(&sched[2 + tid], s_cost[tid]);
+    __threadfence();
+  }
+  __syncthreads();
+  if (tid == 0) {
+    bases[blockIdx.x] = agg;
+    __threadfence();
+    s_last = atomicAdd(reinterpret_cast<uint32_t*>(total + kTotalTicket), 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  uint64_t carry = 0;
+  for (uint32_t b = 0; b < gridDim.x; b += kBinThreads) {
+    const uint32_t i = b + tid;
+    const uint64_t v = i < gridDim.x ? __ldcg(reinterpret_cast<unsigned long long*>(bases) + i) : 0ull;
+    uint64_t a64;
+    const uint64_t ex = block_exclusive_sum<kBinThreads>(v, s_warp64, &a64);
+    if (i < gridDim.x) bases[i] = ex + carry;
+    carry += a64;
+  }
+  if (sched && tid < 32) {  // kCostBuckets == 33: lane l takes bucket l, the last bucket follows the others
+    const uint32_t v = __ldcg(&sched[2 + tid]);
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (tid >= o) incl += y;
+    }
+    sched[2 + kCostBuckets + tid] = incl - v;
+    if (tid == 31) sched[2 + kCostBuckets + 32] = incl;
+  }
+  if (tid == 0) {
+    total[0] = carry;
+    mirror[0] = carry;
+    mirror[1] = total[1];
+    __threadfence_system();
+  }
+}
+
+// Sorts a[0, n) ascending in place: a bitonic network whose comparators all point up, so that the elements
+// past n (as if infinite) never move. The group of `size` threads that calls it (member `me`) synchronises
+// with `sync`. For lists the bucket sort below cannot split.
+template <typename Sync>
+__device__ __forceinline__ void bitonic_sort(unsigned long long* a, uint32_t n, uint32_t me, uint32_t size, Sync sync) {
+  for (uint32_t k = 2; k != 0 && (k >> 1) < n; k <<= 1) {
+    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+      const uint32_t mask = j == (k >> 1) ? k - 1 : j;  // the first step of a merge mirrors its second half
+      for (uint32_t i = me; i < n; i += size) {
+        const uint32_t p = i ^ mask;
+        if (p > i && p < n) {
+          const unsigned long long x = a[i], y = a[p];
+          if (y < x) {
+            a[i] = y;
+            a[p] = x;
+          }
+        }
+      }
+      sync();
+    }
+  }
+}
+
+// A key's bucket: linear over the list's range of depth bits (or of record indices, where all depths are
+// equal), so that equal keys share one and buckets ascend with the keys.
+struct BucketMap {
+  uint32_t lo;
+  float scale;
+  bool by_id;
+  __device__ __forceinline__ BucketMap(uint32_t hmin, uint32_t hmax, uint32_t lmin, uint32_t lmax, uint32_t nb)
+      : lo(hmin == hmax ? lmin : hmin),
+        scale((float)nb / ((float)(hmin == hmax ? lmax - lmin : hmax - hmin) + 1.0f)),
+        by_id(hmin == hmax) {}
+  __device__ __forceinline__ uint32_t operator()(unsigned long long key, uint32_t nb) const {
+    const uint32_t v = (by_id ? (uint32_t)key : (uint32_t)(key >> 32)) - lo;
+    return min((uint32_t)(__uint2float_rz(v) * scale), nb - 1);
+  }
+};
+
+// The position of key a[i] among the keys of its bucket a[first, last).
+__device__ __forceinline__ uint32_t rank_in_bucket(const unsigned long long* a, uint32_t first, uint32_t last,
+                                                   unsigned long long key) {
+  uint32_t r = first;
+  if (last - first > 1)
+    for (uint32_t q = first; q < last; ++q) r += a[q] < key ? 1u : 0u;
+  return r;
+}
+
+// One warp sorts keys[0, n), n <= kWarpList, and writes the record indices to out. One bucket per key or more:
+// count, scan, scatter into shared memory, then each key's place within its bucket by comparison.
+__device__ __forceinline__ void warp_sort_list(const unsigned long long* __restrict__ keys, uint32_t n,
+                                               uint32_t* __restrict__ out, unsigned long long* s_key, uint32_t* s_cnt) {
+  constexpr int kPer = kWarpList / 32;
+  const uint32_t full = 0xFFFFFFFFu, lane = threadIdx.x & 31;
+  unsigned long long k[kPer];
+  uint32_t hmin = full, hmax = 0, lmin = full, lmax = 0;
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    if (j * 32u >= n) break;
+    if (j * 32 + lane < n) {
+      k[j] = keys[j * 32 + lane];
+      hmin = min(hmin, (uint32_t)(k[j] >> 32));
+      hmax = max(hmax, (uint32_t)(k[j] >> 32));
+      lmin = min(lmin, (uint32_t)k[j]);
+      lmax = max(lmax, (uint32_t)k[j]);
+    }
+  }
+  hmin = __reduce_min_sync(full, hmin);
+  hmax = __reduce_max_sync(full, hmax);
+  if (hmin == hmax) {
+    lmin = __reduce_min_sync(full, lmin);
+    lmax = __reduce_max_sync(full, lmax);
+  }
+  const BucketMap bucket(hmin, hmax, lmin, lmax, kWarpBuckets);
+  uint4* cnt4 = reinterpret_cast<uint4*>(s_cnt);
+  cnt4[2 * lane] = cnt4[2 * lane + 1] = make_uint4(0, 0, 0, 0);
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    if (j * 32u >= n) break;
+    if (j * 32 + lane < n) atomicAdd(&s_cnt[bucket(k[j], kWarpBuckets)], 1u);
+  }
+  __syncwarp();
+  uint4 c0 = cnt4[2 * lane], c1 = cnt4[2 * lane + 1];
+  const uint32_t most = __reduce_max_sync(full, max(max(max(c0.x, c0.y), max(c0.z, c0.w)), max(max(c1.x, c1.y), max(c1.z, c1.w))));
+  const uint32_t sum = c0.x + c0.y + c0.z + c0.w + c1.x + c1.y + c1.z + c1.w;
+  uint32_t run = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(full, run, o);
+    if (lane >= (uint32_t)o) run += y;
+  }
+  run -= sum;
+  uint4 e0, e1;
+  e0.x = run;
+  e0.y = e0.x + c0.x;
+  e0.z = e0.y + c0.y;
+  e0.w = e0.z + c0.z;
+  e1.x = e0.w + c0.w;
+  e1.y = e1.x + c1.x;
+  e1.z = e1.y + c1.y;
+  e1.w = e1.z + c1.z;
+  cnt4[2 * lane] = e0;
+  cnt4[2 * lane + 1] = e1;
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    if (j * 32u >= n) break;
+    if (j * 32 + lane < n) s_key[atomicAdd(&s_cnt[bucket(k[j], kWarpBuckets)], 1u)] = k[j];
+  }
+  __syncwarp();  // s_cnt[b] is now the end of bucket b
+  if (most > kHeavy) {
+    bitonic_sort(s_key, n, lane, 32, [] { __syncwarp(); });
+    for (uint32_t i = lane; i < n; i += 32) out[i] = (uint32_t)s_key[i];
+  } else {
+    for (uint32_t i = lane; i < n; i += 32) {
+      const unsigned long long key = s_key[i];
+      const uint32_t b = bucket(key, kWarpBuckets);
+      out[rank_in_bucket(s_key, b ? s_cnt[b - 1] : 0u, s_cnt[b], key)] = (uint32_t)key;
+    }
+  }
+}
+
+// Exclusive prefix sums of the CTA's kCtaBuckets counts, in place; the largest count is returned to every thread.
+__device__ __forceinline__ uint32_t cta_scan_buckets(uint32_t* s_cnt, uint32_t* s_red) {
+  const uint32_t tid = threadIdx.x;
+  uint4* cnt4 = reinterpret_cast<uint4*>(s_cnt);
+  const uint4 c0 = cnt4[2 * tid], c1 = cnt4[2 * tid + 1];
+  uint32_t most = max(max(max(c0.x, c0.y), max(c0.z, c0.w)), max(max(c1.x, c1.y), max(c1.z, c1.w)));
+  most = __reduce_max_sync(0xFFFFFFFFu, most);
+  if ((tid & 31) == 0) s_red[8 + (tid >> 5)] = most;
+  const uint32_t sum = c0.x + c0.y + c0.z + c0.w + c1.x + c1.y + c1.z + c1.w;
+  uint32_t agg;
+  const uint32_t run = block_exclusive_sum<kSortThreads>(sum, s_red, &agg);
+#pragma unroll
+  for (int w = 0; w < kSortThreads / 32; ++w) most = max(most, s_red[8 + w]);
+  uint4 e0, e1;
+  e0.x = run;
+  e0.y = e0.x + c0.x;
+  e0.z = e0.y + c0.y;
+  e0.w = e0.z + c0.z;
+  e1.x = e0.w + c0.w;
+  e1.y = e1.x + c1.x;
+  e1.z = e1.y + c1.y;
+  e1.w = e1.z + c1.z;
+  cnt4[2 * tid] = e0;
+  cnt4[2 * tid + 1] = e1;
+  __syncthreads();
+  return most;
+}
+
+// The range of the CTA's keys (each thread has reduced its own), and zeroed bucket counts.
+__device__ __forceinline__ BucketMap cta_bucket_map(uint32_t hmin, uint32_t hmax, uint32_t lmin, uint32_t lmax,
+                                                    uint32_t* s_cnt, uint32_t* s_red) {
+  const uint32_t full = 0xFFFFFFFFu, tid = threadIdx.x, warp = tid >> 5;
+  hmin = __reduce_min_sync(full, hmin);
+  hmax = __reduce_max_sync(full, hmax);
+  lmin = __reduce_min_sync(full, lmin);
+  lmax = __reduce_max_sync(full, lmax);
+  __syncthreads();  // the previous list's use of the shared arrays is over
+  if ((tid & 31) == 0) {
+    s_red[warp] = hmin;
+    s_red[8 + warp] = hmax;
+    s_red[16 + warp] = lmin;
+    s_red[24 + warp] = lmax;
+  }
+  uint4* cnt4 = reinterpret_cast<uint4*>(s_cnt);
+  cnt4[2 * tid] = cnt4[2 * tid + 1] = make_uint4(0, 0, 0, 0);
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kSortThreads / 32; ++w) {
+    hmin = min(hmin, s_red[w]);
+    hmax = max(hmax, s_red[8 + w]);
+    lmin = min(lmin, s_red[16 + w]);
+    lmax = max(lmax, s_red[24 + w]);
+  }
+  return BucketMap(hmin, hmax, lmin, lmax, kCtaBuckets);
+}
+
+// The keys of a run of buckets stand in s_key[0, m), the run starting at list position `first`; s_cnt holds each
+// bucket's end. Writes their record indices in order.
+__device__ __forceinline__ void cta_write_run(unsigned long long* s_key, const uint32_t* s_cnt, uint32_t m, uint32_t first,
+                                              const BucketMap& bucket, bool heavy, uint32_t* __restrict__ out) {
+  if (heavy) {
+    bitonic_sort(s_key, m, threadIdx.x, kSortThreads, [] { __syncthreads(); });
+    for (uint32_t i = threadIdx.x; i < m; i += kSortThreads) out[first + i] = (uint32_t)s_key[i];
+    return;
+  }
+  for (uint32_t i = threadIdx.x; i < m; i += kSortThreads) {
+    const unsigned long long key = s_key[i];
+    const uint32_t b = bucket(key, kCtaBuckets);
+    const uint32_t from = b ? s_cnt[b - 1] : 0u;
+    out[first + rank_in_bucket(s_key, from - first, s_cnt[b] - first, key)] = (uint32_t)key;
+  }
+}
+
+// A CTA sorts keys[0, n), n <= kCtaList, as the warps do; the keys stay in registers between the passes.
+__device__ __forceinline__ void cta_sort_list(const unsigned long long* __restrict__ keys, uint32_t n,
+                                              uint32_t* __restrict__ out, unsigned long long* s_key, uint32_t* s_cnt,
+                                              uint32_t* s_red) {
+  constexpr int kPer = kCtaList / kSortThreads;
+  const uint32_t full = 0xFFFFFFFFu, tid = threadIdx.x;
+  unsigned long long k[kPer];
+  uint32_t hmin = full, hmax = 0, lmin = full, lmax = 0;
+#pragma unroll
+  for (int j = 0; j < kPer; ++j)
+    if (j * kSortThreads + tid < n) k[j] = keys[j * kSortThreads + tid];
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    if (j * kSortThreads + tid < n) {
+      hmin = min(hmin, (uint32_t)(k[j] >> 32));
+      hmax = max(hmax, (uint32_t)(k[j] >> 32));
+      lmin = min(lmin, (uint32_t)k[j]);
+      lmax = max(lmax, (uint32_t)k[j]);
+    }
+  }
+  const BucketMap bucket = cta_bucket_map(hmin, hmax, lmin, lmax, s_cnt, s_red);
+#pragma unroll
+  for (int j = 0; j < kPer; ++j)
+    if (j * kSortThreads + tid < n) atomicAdd(&s_cnt[bucket(k[j], kCtaBuckets)], 1u);
+  __syncthreads();
+  const uint32_t most = cta_scan_buckets(s_cnt, s_red);
+#pragma unroll
+  for (int j = 0; j < kPer; ++j)
+    if (j * kSortThreads + tid < n) s_key[atomicAdd(&s_cnt[bucket(k[j], kCtaBuckets)], 1u)] = k[j];
+  __syncthreads();
+  cta_write_run(s_key, s_cnt, n, 0, bucket, most > kHeavy, out);
+}
+
+// A list of any length: taken in runs of consecutive buckets that shared memory holds, one reading of the list per
+// run. A bucket that alone exceeds it leaves the list to the network, in place in global memory.
+__device__ __noinline__ void cta_sort_long_list(unsigned long long* keys, uint32_t n, uint32_t* __restrict__ out,
+                                                unsigned long long* s_key, uint32_t* s_cnt, uint32_t* s_red) {
+  const uint32_t full = 0xFFFFFFFFu, tid = threadIdx.x;
+  uint32_t hmin = full, hmax = 0, lmin = full, lmax = 0;
+  for (uint32_t i = tid; i < n; i += kSortThreads) {
+    const unsigned long long k = keys[i];
+    hmin = min(hmin, (uint32_t)(k >> 32));
+    hmax = max(hmax, (uint32_t)(k >> 32));
+    lmin = min(lmin, (uint32_t)k);
+    lmax = max(lmax, (uint32_t)k);
+  }
+  const BucketMap bucket = cta_bucket_map(hmin, hmax, lmin, lmax, s_cnt, s_red);
+  for (uint32_t i = tid; i < n; i += kSortThreads) atomicAdd(&s_cnt[bucket(keys[i], kCtaBuckets)], 1u);
+  __syncthreads();
+  const uint32_t most = cta_scan_buckets(s_cnt, s_red);
+  if (most > (uint32_t)kCtaList) {
+    bitonic_sort(keys, n, tid, kSortThreads, [] { __syncthreads(); });
+    for (uint32_t i = tid; i < n; i += kSortThreads) out[i] = (uint32_t)keys[i];
+    return;
+  }
+  for (uint32_t b0 = 0, first = 0; first < n;) {
+    // buckets [b0, b1) hold at most kCtaList keys, list positions [first, last)
+    uint32_t b1 = kCtaBuckets, last = n;
+    if (n - first > (uint32_t)kCtaList) {
+      uint32_t l = b0 + 1, h = kCtaBuckets - 1;  // start(b0 + 1) - first <= kCtaList: no bucket is larger
+      while (l < h) {
+        const uint32_t mid = (l + h + 1) >> 1;
+        if (s_cnt[mid] - first <= (uint32_t)kCtaList) l = mid;
+        else h = mid - 1;
+      }
+      b1 = l;
+      last = s_cnt[b1];
+    }
+    __syncthreads();  // every thread has read the starts that the scatter advances to the ends
+    for (uint32_t i = tid; i < n; i += kSortThreads) {
+      const unsigned long long k = keys[i];
+      const uint32_t b = bucket(k, kCtaBuckets);
+      if (b >= b0 && b < b1) s_key[atomicAdd(&s_cnt[b], 1u) - first] = k;
+    }
+    __syncthreads();
+    cta_write_run(s_key, s_cnt, last - first, first, bucket, most > kHeavy, out);
+    __syncthreads();
+    b0 = b1;
+    first = last;
+  }
+}
+
+// Tile t's segment of the pair array: an asynchronous render's lists may run past the capacity.
+__device__ __forceinline__ uint2 tile_segment(const uint64_t* __restrict__ bases, uint2 local, uint32_t t, uint32_t cap) {
+  const uint64_t base = bases[t / kBinBlock];
+  const uint2 r = make_uint2((uint32_t)min(base + local.x, (uint64_t)cap), (uint32_t)min(base + local.y, (uint64_t)cap));
+  return r.y > r.x ? r : make_uint2(0, 0);
+}
+
+// Sorts every tile's segment and finishes its range: [start, end), or (0, 0) for an empty tile. The first
+// `big_ctas` CTAs take the lists of more than kWarpList keys (from `big`, or, where that overflowed, among all
+// tiles), each sorted by the whole CTA; the warps of the others take one tile each. With `sched`, each tile takes
+// its place in the work list of descending cost.
+__global__ void __launch_bounds__(kSortThreads, 5)
+    tile_sort_kernel(unsigned long long* keys, uint32_t cap, const uint64_t* __restrict__ bases, uint32_t ntiles,
+                     const uint2* local, uint2* __restrict__ ranges, uint32_t* __restrict__ out, uint32_t big_ctas,
+                     const uint32_t* __restrict__ big, uint32_t big_cap, const uint64_t* __restrict__ total,
+                     uint32_t* __restrict__ sched, uint32_t* __restrict__ work) {
+  pdl_wait();
+  __shared__ __align__(16) unsigned long long s_key[kCtaList];
+  __shared__ __align__(16) uint32_t s_cnt[kCtaBuckets];
+  __shared__ uint32_t s_red[32];
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto finish = [&](uint32_t t, uint2 l, uint2 r) {  // by one thread, after the tile's offsets have been read
+    ranges[t] = r;
+    // the cost bucket counted by the scan: the whole list, also where the capacity cuts it
+    if (sched) work[atomicAdd(&sched[2 + kCostBuckets + cost_bucket(l)], 1u)] = t;
+  };
+  if (blockIdx.x < big_ctas) {
+    const uint32_t listed = (uint32_t)total[kTotalBig];
+    const uint32_t items = listed <= big_cap ? listed : ntiles;
+    for (uint32_t i = blockIdx.x; i < items; i += big_ctas) {
+      const uint32_t t = listed <= big_cap ? big[i] : i;
+      const uint2 l = local[t];
+      if (l.y - l.x <= (uint32_t)kWarpList) continue;
+      const uint2 r = tile_segment(bases, l, t, cap);
+      const uint32_t n = r.y - r.x;
+      if (n > (uint32_t)kCtaList) cta_sort_long_list(keys + r.x, n, out + r.x, s_key, s_cnt, s_red);
+      else if (n) cta_sort_list(keys + r.x, n, out + r.x, s_key, s_cnt, s_red);
+      __syncthreads();
+      if (threadIdx.x == 0) finish(t, l, r);
+    }
+    return;
+  }
+  const uint32_t t = (blockIdx.x - big_ctas) * (kSortThreads / 32) + warp;
+  if (t >= ntiles) return;
+  const uint2 l = local[t];
+  __syncwarp();  // lane 0 overwrites it below
+  if (l.y - l.x > (uint32_t)kWarpList) return;
+  const uint2 r = tile_segment(bases, l, t, cap);
+  const uint32_t n = r.y - r.x;
+  if (n > 1)
+    warp_sort_list(keys + r.x, n, out + r.x, s_key + warp * kWarpList, s_cnt + warp * kWarpBuckets);
+  else if (n == 1 && lane == 0)
+    out[r.x] = (uint32_t)keys[r.x];
+  if (lane == 0) finish(t, l, r);
 }
 
 }  // namespace
@@ -469,11 +897,28 @@ void launch_tile_ranges(const uint32_t* tiles, const uint32_t* vals, const ViewP
              npairs_cap, npairs_dev, ntiles, ranges, check);
 }
 
-void launch_compose_keys(const uint32_t* tiles, const uint32_t* vals, const float4* rec, const ViewParams* views,
-                         uint32_t n_per_view, uint32_t n_views, uint32_t npairs, uint64_t* keys, cudaStream_t s) {
-  if (npairs == 0) return;
-  compose_keys_kernel<<<(npairs + 255) / 256, 256, 0, s>>>(tiles, vals, rec, views, n_per_view, n_views, npairs,
-                                                           keys);
+void launch_compose_keys(const uint2* ranges, uint32_t ntiles, const uint32_t* ids, const float4* rec, uint64_t* keys,
+                         cudaStream_t s) {
+  if (ntiles == 0) return;
+  compose_keys_kernel<<<(ntiles + 7) / 8, 256, 0, s>>>(ranges, ntiles, ids, rec, keys);
+}
+
+size_t bin_bases_words(uint64_t ntiles) { return (size_t)((ntiles + kBinBlock - 1) / kBinBlock); }
+
+void launch_tile_scan(uint2* ranges, uint32_t ntiles, uint64_t* bases, uint64_t* total, uint32_t* big, uint32_t big_cap,
+                      uint32_t* sched, uint64_t* mirror, cudaStream_t s) {
+  launch_pdl(tile_scan_kernel, (ntiles + kBinBlock - 1) / kBinBlock, kBinThreads, 0, s, ranges, ntiles, bases, total, big,
+             big_cap, sched, mirror);
+}
+
+void launch_tile_sort(uint64_t* keys, uint32_t cap, const uint64_t* bases, uint32_t ntiles, uint2* ranges, uint32_t* out,
+                      const uint32_t* big, uint32_t big_cap, const uint64_t* total, uint32_t* sched, uint32_t* work,
+                      int num_sms, cudaStream_t s) {
+  constexpr uint32_t kTiles = kSortThreads / 32;
+  const uint32_t big_ctas = std::min(ntiles, 4u * (uint32_t)std::max(num_sms, 1));  // one wave
+  launch_pdl(tile_sort_kernel, big_ctas + (ntiles + kTiles - 1) / kTiles, kSortThreads, 0, s,
+             reinterpret_cast<unsigned long long*>(keys), cap, bases, ntiles, ranges, ranges, out, big_ctas, big, big_cap,
+             total, sched, work);
 }
 
 }  // namespace ngs
