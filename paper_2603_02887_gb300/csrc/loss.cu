@@ -16,7 +16,8 @@
 // rows, and each thread then convolves one column vertically for four output rows. Pairs of values (x and y, their
 // squares) go through packed FP32x2 instructions together. Only a / b / c pass through memory (36 B per pixel), where
 // four separable passes moved 24 planes of moments and partials; every sum has the order of those passes.
-// 282 -> 80 us at 1920 x 1080 on GB300.
+// 282 -> 144 us at 1920 x 1080 on GB300 (map 76, gradient 68), bound by FP32 issue: seven IEEE divisions per channel
+// of a pixel are half of the map's instructions.
 #include <math.h>
 #include <string.h>
 
@@ -265,10 +266,13 @@ __global__ void __launch_bounds__(kLossThreads, 4)
     __syncthreads();
     const int out0 = in0 - 6;
     if (step < 3 || tid >= kOutThreads || x0 + vx >= W) continue;
-    float2 t[kRows];
+    const size_t at0 = ((size_t)out0 * W + x0) * 3 + tid;
+    float2 t[kRows], xy[kRows];  // (the pixels are on their way during the convolution)
     float e[kRows];
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
+      const size_t at = at0 + (size_t)r * 3 * W;
+      xy[r] = out0 + r < H ? make_float2(x[at], y[at]) : make_float2(0.f, 0.f);
       t[r] = make_float2(0.f, 0.f);
       e[r] = 0.f;
     }
@@ -288,12 +292,11 @@ __global__ void __launch_bounds__(kLossThreads, 4)
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
       if (out0 + r >= H) break;
-      const size_t at = ((size_t)(out0 + r) * W + x0) * 3 + tid;
-      const float a = x[at], b = y[at];
+      const float a = xy[r].x, b = xy[r].y;
       const float dssim = t[r].x + 2.f * a * t[r].y + b * e[r];
       const float d = a - b;
       const float sgn = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
-      dl[at] = w_l1 * sgn - w_ssim * dssim;
+      dl[at0 + (size_t)r * 3 * W] = w_l1 * sgn - w_ssim * dssim;
     }
   }
 }
