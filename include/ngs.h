@@ -101,7 +101,8 @@ typedef struct {
   int32_t max_splats;  /* 0 = unlimited, else at most this many splats composited per pixel (the    */
                        /* paper's ray tracer caps at 128, Sec. 5.1 "Renderer")                       */
   int32_t chunk;       /* splat records staged in shared memory per round of a tile's list walk:      */
-                       /* 0 = the tile's pixel count (default), else half, equal to or twice it       */
+                       /* 0 = the tile's pixel count or half of it (default: chosen by model and      */
+                       /* frame size), else half, equal to or twice it                                */
   int32_t schedule;    /* NGS_SCHEDULE_TILES (default) or NGS_SCHEDULE_PERSISTENT                     */
 } ngs_options;         /* tile shape, chunk and schedule change the speed, never the results          */
 

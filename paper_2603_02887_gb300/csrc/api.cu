@@ -414,7 +414,7 @@ static cudaError_t phase2(ngs_ctx* ctx, ngs_frame* f, const RenderPlan& pl, uint
     stage_begin(ctx, s, 3, &ev);
     f->p_final = 0;
     launch_tile_sort(f->ptiles.as<uint64_t>(), cap, ctx->scan_tmp.as<uint64_t>(), pl.ntiles, f->ranges.as<uint2>(),
-                     f->pvals[0].as<uint32_t>(), f->offsets.as<uint32_t>(), pl.R + 1, ctx->total.as<uint64_t>(), counter,
+                     f->pvals[0].as<uint32_t>(), f->pvals[1].as<uint32_t>(), f->offsets.as<uint32_t>(), pl.R + 1, ctx->total.as<uint64_t>(), counter,
                      f->work.as<uint32_t>(), ctx->num_sms, s);
     stage_end(ctx, s, 3, ev, 1);
   } else {
@@ -529,6 +529,41 @@ static int run_phase(ngs_ctx* ctx, ngs_frame* f, int which, const KeyBuf& key, c
   return NGS_OK;
 }
 
+// Phase 2 for `cap` pairs (a graph replay while its launch arguments are unchanged).
+static int enqueue_phase2(ngs_ctx* ctx, ngs_frame* f, const RenderPlan& pl, int n_views, uint32_t cap,
+                          const uint32_t* np_dev, bool async, cudaStream_t s) {
+  KeyBuf k2;
+  k2.add(pl.rp);
+  k2.add(cap);
+  k2.add(np_dev);
+  k2.add(async);
+  k2.add(f->g_final);
+  k2.add(n_views == 1 ? pl.image : nullptr);  // a batch reads its outputs from the view table
+  k2.add(n_views == 1 ? pl.overdraw : nullptr);
+  k2.add(ctx->num_sms);
+  for (const ViewParams& vp : f->view_host) {  // the tile sort's bit count follows the largest view
+    k2.add(vp.tiles_x);
+    k2.add(vp.tiles_y);
+  }
+  for (const DevBuf* b : {&f->rec, &f->gkeys[0], &f->gkeys[1], &f->gvals[0], &f->gvals[1], &f->offsets, &f->views,
+                          &f->ptiles, &f->tile_count, &ctx->total, &f->pvals[0], &f->pvals[1], &ctx->hist,
+                          &ctx->scan_tmp, &f->ranges, &f->work, &f->sched, &f->state})
+    k2.add(b->p);
+  if (async) k2.add(f->d_status);
+  return run_phase(ctx, f, 1, k2, s, [&](cudaStream_t st) { return phase2(ctx, f, pl, cap, np_dev, async, st); });
+}
+
+// Records staged per round when the caller leaves it open: the tile's pixel count. On frames of many tiles of 256 pixels
+// or more, half of it for the models whose kernels walk two pixels per thread: a tile whose rays have all stopped has
+// then loaded fewer records past the stop, and more CTAs fit an SM (render + backward at 500k Gaussians, 1920x1080,
+// c = +0.5: 415 -> 388 us; 1M, 1297x840, c = 0: 564 -> 544). With few tiles the shorter rounds only add waits (1k
+// Gaussians, 128x128: 87 -> 90 us).
+constexpr uint64_t kManyTiles = 2048;
+static int default_chunk(int kind, int pixels, uint64_t ntiles) {
+  const bool pairs = kind == NGS_MODEL_EXP || kind == NGS_MODEL_QUAD;
+  return pairs && pixels >= 256 && ntiles >= kManyTiles ? pixels / 2 : pixels;
+}
+
 // The render pipeline for n_views cameras of one set of Gaussians (n_views = 1 for ngs_render).
 int ngs::render_views(ngs_ctx* ctx, ngs_frame* f, const ngs_gaussians* g, const ngs_camera* cams, int n_views,
                       const ngs_model* model, const ngs_options* o, float* image, int32_t* overdraw,
@@ -606,7 +641,7 @@ int ngs::render_views_out(ngs_ctx* ctx, ngs_frame* f, const ngs_gaussians* g, co
   rp.width = cams[0].width;
   rp.height = cams[0].height;
   rp.max_splats = o->max_splats;
-  rp.chunk = o->chunk ? o->chunk : o->tile_w * o->tile_h;
+  rp.chunk = o->chunk ? o->chunk : default_chunk(model->kind, o->tile_w * o->tile_h, tiles_total);
   rp.schedule = o->schedule;
   rp.sh_degree = g->sh_degree;
   rp.n_gaussians = (uint32_t)g->n;
@@ -676,18 +711,40 @@ int ngs::render_views_out(ngs_ctx* ctx, ngs_frame* f, const ngs_gaussians* g, co
   k1.add(ctx->h_total);
   // asynchronous: no host synchronisation; phase 2 is sized by the frame's capacity (set by earlier renders)
   const bool async = f->async && f->pair_cap > 0 && !admit;
-  NGS_TRY(run_phase(ctx, f, 0, k1, s, [&](cudaStream_t st) { return phase1(ctx, f, pl, st); }));
-  cudaError_t e = cudaEventRecord(f->views_uploaded, s);
+  // Otherwise the host needs the pair count. Where the frame already holds pair buffers and the lists are built by
+  // counting (no launch of phase 2 then depends on the count), phase 2 is enqueued for what the buffers hold before the
+  // host waits, so that the GPU does not idle meanwhile: an idle of about 12 us per render. A count that does not fit is
+  // met on the old path: both phases once more, with the exact count.
+  uint32_t spec = 0;
+  if (!async && !admit && pl.bins && f->pair_cap > 0)
+    spec = (uint32_t)std::min<uint64_t>(std::min(f->ptiles.cap / 8, f->pvals[0].cap / 4), (1ull << 31) - 1);
+  if (ctx->graphs && spec < f->pair_cap) spec = 0;  // (a graph is captured for the capacity)
+  if (ctx->graphs && spec) spec = f->pair_cap;
+  const uint32_t* const count_dev = reinterpret_cast<const uint32_t*>(ctx->total.p);  // low word of the pair count (< 2^31)
+  cudaError_t e = cudaSuccess;
   uint32_t np = 0, cap = 0;
   const uint32_t* np_dev = nullptr;
-  if (async) {
-    if (e != cudaSuccess) return fail(ctx, NGS_ERR_CUDA, std::string("render: ") + cudaGetErrorString(e));
-    cap = f->pair_cap;
-    np_dev = reinterpret_cast<const uint32_t*>(ctx->total.p);  // low word of the pair count (< 2^31)
-  } else {
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  for (bool again = false;; again = true) {
+    NGS_TRY(run_phase(ctx, f, 0, k1, s, [&](cudaStream_t st) { return phase1(ctx, f, pl, st); }));
+    e = cudaEventRecord(f->views_uploaded, s);
+    if (async) {
+      if (e != cudaSuccess) return fail(ctx, NGS_ERR_CUDA, std::string("render: ") + cudaGetErrorString(e));
+      cap = f->pair_cap;
+      np_dev = count_dev;
+      break;
+    }
+    if (spec && !again) {
+      if (e != cudaSuccess) return fail(ctx, NGS_ERR_CUDA, std::string("render: ") + cudaGetErrorString(e));
+      NGS_TRY(enqueue_phase2(ctx, f, pl, n_views, spec, ctx->graphs ? count_dev : nullptr, false, s));
+      e = cudaEventSynchronize(f->views_uploaded);
+    } else if (e == cudaSuccess) {
+      e = cudaStreamSynchronize(s);
+    }
     if (e != cudaSuccess) return fail(ctx, NGS_ERR_CUDA, std::string("reading the pair count: ") + cudaGetErrorString(e));
-    const volatile uint64_t* mirror = ctx->h_total + kMirrorTotal;  // written by publish_words
+    const volatile uint64_t* mirror = ctx->h_total + kMirrorTotal;  // written at the end of phase 1
+    // an error return leaves nothing behind that would still write the caller's memory
+    if (spec && !again && (mirror[1] != 0 || mirror[0] >= (1ull << 31)) && (e = cudaStreamSynchronize(s)) != cudaSuccess)
+      return fail(ctx, NGS_ERR_CUDA, std::string("render: ") + cudaGetErrorString(e));
     if (mirror[1] != 0) {  // a bounds check fired in an earlier call on this context
       const cudaError_t ze = cudaMemsetAsync(ctx->total.as<uint64_t>() + 1, 0, sizeof(uint64_t), s);
       if (ze != cudaSuccess)
@@ -703,37 +760,23 @@ int ngs::render_views_out(ngs_ctx* ctx, ngs_frame* f, const ngs_gaussians* g, co
                                                                  rp.schedule, np))));
     // the capacity that graph replays and asynchronous renders reuse while the count fits
     if (np > f->pair_cap) f->pair_cap = (uint32_t)std::min<uint64_t>((uint64_t)np + np / 4 + 1024, (1ull << 31) - 1);
+    if (spec && !again && np > spec) continue;
     // phase 2: exact sizes, or, for graph replays, the capacity
     cap = np;
     if (ctx->graphs) {
       cap = f->pair_cap;
-      np_dev = reinterpret_cast<const uint32_t*>(ctx->total.p);
+      np_dev = count_dev;
     }
+    if (again) spec = 0;
+    break;
   }
-  const BufferPlan bp2 = plan_buffers(R, pl.n, (uint32_t)n_views, pl.ntiles, pix_total, rp.schedule, cap);
-  NGS_TRY(ensure(ctx, f->ptiles, pair_keys_bytes(bp2)));
-  for (int k = 0; k < 2; ++k) NGS_TRY(ensure(ctx, f->pvals[k], bp2.pair_val));
-  NGS_TRY(ensure(ctx, ctx->hist, bp2.hist2));
-  KeyBuf k2;
-  k2.add(rp);
-  k2.add(cap);
-  k2.add(np_dev);
-  k2.add(async);
-  k2.add(f->g_final);
-  k2.add(n_views == 1 ? pl.image : nullptr);  // a batch reads its outputs from the view table
-  k2.add(n_views == 1 ? pl.overdraw : nullptr);
-  k2.add(ctx->num_sms);
-  for (const ViewParams& vp : f->view_host) {  // the tile sort's bit count follows the largest view
-    k2.add(vp.tiles_x);
-    k2.add(vp.tiles_y);
+  if (!spec) {
+    const BufferPlan bp2 = plan_buffers(R, pl.n, (uint32_t)n_views, pl.ntiles, pix_total, rp.schedule, cap);
+    NGS_TRY(ensure(ctx, f->ptiles, pair_keys_bytes(bp2)));
+    for (int k = 0; k < 2; ++k) NGS_TRY(ensure(ctx, f->pvals[k], bp2.pair_val));
+    NGS_TRY(ensure(ctx, ctx->hist, bp2.hist2));
+    NGS_TRY(enqueue_phase2(ctx, f, pl, n_views, cap, np_dev, async, s));
   }
-  for (const DevBuf* b : {&f->rec, &f->gkeys[0], &f->gkeys[1], &f->gvals[0], &f->gvals[1], &f->offsets, &f->views,
-                          &f->ptiles, &f->tile_count, &ctx->total,
-                          &f->pvals[0], &f->pvals[1], &ctx->hist, &ctx->scan_tmp, &f->ranges, &f->work, &f->sched,
-                          &f->state})
-    k2.add(b->p);
-  if (async) k2.add(f->d_status);
-  NGS_TRY(run_phase(ctx, f, 1, k2, s, [&](cudaStream_t st) { return phase2(ctx, f, pl, cap, np_dev, async, st); }));
   if (async) {
     e = cudaEventRecord(f->done, s);
     if (e != cudaSuccess) return fail(ctx, NGS_ERR_CUDA, std::string("render: ") + cudaGetErrorString(e));

@@ -393,9 +393,10 @@ void launch_emit_bins(const float4* rec, const uint32_t* tile_count, const TileM
                       const RenderParams& rp, uint2* ranges, const uint64_t* bases, uint64_t* keys, uint32_t cap,
                       cudaStream_t s);
 // Sorts each tile's segment of keys; the record indices go to out, the final [start, end) to ranges, and (with
-// sched) the tiles to the work list of the persistent schedule. The segments of keys are scratch afterwards.
+// sched) the tiles to the work list of the persistent schedule. The segments of keys are scratch afterwards; `tmp` (cap words) is
+// scratch for the longest lists.
 void launch_tile_sort(uint64_t* keys, uint32_t cap, const uint64_t* bases, uint32_t ntiles, uint2* ranges, uint32_t* out,
-                      const uint32_t* big, uint32_t big_cap, const uint64_t* total, uint32_t* sched, uint32_t* work,
+                      uint32_t* tmp, const uint32_t* big, uint32_t big_cap, const uint64_t* total, uint32_t* sched, uint32_t* work,
                       int num_sms, cudaStream_t s);
 // [start, end) of every global tile's pairs into `ranges`, which the caller has zeroed (zero-length ranges
 // stay (0, 0)); npairs_cap items are covered by the grid, of which the first *npairs_dev are valid if

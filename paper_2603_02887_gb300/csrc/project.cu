@@ -349,23 +349,60 @@ __device__ __forceinline__ void add_to_bins(uint2* bins, const RenderParams& rp,
   for (int tx = t0; tx <= t1; ++tx) atomicAdd(&b[tx].y, 1u);
 }
 
-// Tiles covered over tile rows [y0, y1] (columns clipped to [x0, x1]), added to the tiles' counts if `bins`; mask:
-// their bits in the box's 8 x 8 tiles (columns past the eighth are left out: the caller discards it then).
+// Tiles covered over tile rows [y0, y1] (columns clipped to [x0, x1]).
 __device__ __forceinline__ uint32_t count_rows(const SplatBin& b, const RenderParams& rp, int x0, int x1, int y0,
-                                               int y1, uint2* bins, uint2& mask) {
+                                               int y1) {
   uint32_t c = 0;
   for (int ty = y0; ty <= y1; ++ty) {
     int t0, t1;
-    if (!row_span(b, rp, ty, x0, x1, t0, t1)) continue;
-    c += (uint32_t)(t1 - t0 + 1);
-    if (bins) {
-      add_to_bins(bins, rp, ty, t0, t1);
-      const uint32_t bits = (((2u << min(t1 - x0, 7)) - (1u << min(t0 - x0, 7))) & 0xFFu) << (8 * ((ty - y0) & 3));
-      if (ty - y0 < 4) mask.x |= bits;
-      else mask.y |= bits;
-    }
+    if (row_span(b, rp, ty, x0, x1, t0, t1)) c += (uint32_t)(t1 - t0 + 1);
   }
   return c;
+}
+
+// Counting into bins: the tile rows of a warp's splats (boxes of at most 8 x 8 tiles), listed in shared memory and taken
+// one per lane, whatever splat they belong to. A row costs about a hundred instructions (two square roots and two
+// divisions of exact rounding); with a lane walking the rows of its own splat, the warp waited for its tallest splat:
+// about 8 rows' time for 3 rows of work.
+struct RowList {
+  float4 p[3][32];     // (u, v, A', B'), (C', Tm, dymax, dyr), (x0, x1, y0, -)
+  uint16_t item[256];  // lane | row << 5
+  uint8_t mask[32][8];  // covered tiles of each row of the box
+};
+
+__device__ __forceinline__ uint2 count_listed(RowList& list, const SplatBin& b, const RenderParams& rp, bool small, int x0,
+                                              int x1, int y0, int y1, uint2* bins) {
+  const uint32_t full = 0xFFFFFFFFu;
+  const int lane = threadIdx.x & 31, rows = small ? y1 - y0 + 1 : 0;
+  int off = rows;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(full, off, o);
+    if (lane >= o) off += y;
+  }
+  const int total = __shfl_sync(full, off, 31);
+  off -= rows;
+  list.p[0][lane] = make_float4(b.u, b.v, b.A, b.B);
+  list.p[1][lane] = make_float4(b.C, b.Tm, b.dymax, b.dyr);
+  list.p[2][lane] = make_float4(__int_as_float(x0), __int_as_float(x1), __int_as_float(y0), 0.f);
+  for (int k = 0; k < rows; ++k) list.item[off + k] = (uint16_t)(lane | k << 5);
+  uint2* const my_mask = reinterpret_cast<uint2*>(list.mask[lane]);
+  *my_mask = make_uint2(0, 0);
+  __syncwarp();
+  for (int i = lane; i < total; i += 32) {
+    const int e = list.item[i], src = e & 31, k = e >> 5;
+    const float4 p0 = list.p[0][src], p1 = list.p[1][src], p2 = list.p[2][src];
+    SplatBin c;
+    c.u = p0.x, c.v = p0.y, c.A = p0.z, c.B = p0.w;
+    c.C = p1.x, c.Tm = p1.y, c.dymax = p1.z, c.dyr = p1.w;
+    const int cx0 = __float_as_int(p2.x), ty = __float_as_int(p2.z) + k;
+    int t0, t1;
+    if (!row_span(c, rp, ty, cx0, __float_as_int(p2.y), t0, t1)) continue;
+    list.mask[src][k] = (uint8_t)((2u << (t1 - cx0)) - (1u << (t0 - cx0)));
+    add_to_bins(bins, rp, ty, t0, t1);
+  }
+  __syncwarp();
+  return *my_mask;
 }
 
 // A splat spanning more tile rows than this has them counted by its whole warp, one row per lane.
@@ -375,7 +412,7 @@ constexpr int kCoopRows = 8;  // (the rows of a tile mask)
 // Gaussians run side by side, so their parameters are read from HBM once and from L2 afterwards.
 // A single view takes its camera from the kernel parameters (cam0), a batch (or a captured graph, which
 // must serve any pose) from the view table; the arithmetic below is the same code either way.
-template <int DEG, bool VEC>
+template <int DEG, bool VEC, bool BINS>
 __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const ViewParams* __restrict__ views,
                                                       CamParams cam0, RenderParams rp, float4* rec,
                                                       uint32_t* depth_key, uint32_t* tile_count, uint32_t* order,
@@ -387,7 +424,7 @@ __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const 
   if (rp.n_views != 1) {  // the block's view (one per block)
     rp.tiles_x = views[view].tiles_x;
     rp.tiles_y = views[view].tiles_y;
-    if (bins) bins += views[view].tile_base;
+    if constexpr (BINS) bins += views[view].tile_base;
   }
   const int64_t r = (int64_t)view * g.n + i;  // record index
   if (i < g.n) {
@@ -405,7 +442,7 @@ __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const 
   }
   // every lane stays to the end: the warp counts its tall splats' tiles together
   uint32_t count = 0;
-  bool tall = false;
+  bool tall = false, boxed = false;
   int x0 = 0, x1 = -1, y0 = 0, y1 = -1;
   uint2 mask = make_uint2(0, 0);
   SplatBin b = {};
@@ -434,15 +471,22 @@ __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const 
         r2 = make_float4(E2, z, rx, ry);
         if (tile_rect(r0.x, r0.y, r2.z, r2.w, rp, x0, x1, y0, y1)) {
           b = splat_bin(r0, r1, rp.log2_alpha_min);
-          tall = y1 - y0 >= kCoopRows;
-          if (!tall) count = count_rows(b, rp, x0, x1, y0, y1, bins, mask);
+          tall = y1 - y0 >= kCoopRows || (BINS && x1 - x0 >= 8);
+          boxed = !tall;
+          if constexpr (!BINS)
+            if (!tall) count = count_rows(b, rp, x0, x1, y0, y1);
         }
       }
     }
     rec[3 * r] = r0;
     rec[3 * r + 1] = r1;
     rec[3 * r + 2] = r2;
-    if (!bins) order[r] = (uint32_t)r;
+    if constexpr (!BINS) order[r] = (uint32_t)r;
+  }
+  if constexpr (BINS) {
+    __shared__ __align__(16) RowList s_rows[8];
+    mask = count_listed(s_rows[threadIdx.x >> 5], b, rp, boxed, x0, x1, y0, y1, bins);
+    count = (uint32_t)(__popc(mask.x) + __popc(mask.y));
   }
   // tall splats, one after another: lane l counts tile rows y0 + l, y0 + l + 32, ... (the same row spans)
   for (uint32_t pending = __ballot_sync(0xFFFFFFFFu, tall); pending != 0u; pending &= pending - 1u) {
@@ -463,16 +507,16 @@ __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const 
       int t0, t1;
       if (!row_span(cb, rp, ty, cx0, cx1, t0, t1)) continue;
       c += (uint32_t)(t1 - t0 + 1);
-      if (bins) add_to_bins(bins, rp, ty, t0, t1);
+      if constexpr (BINS) add_to_bins(bins, rp, ty, t0, t1);
     }
     c = __reduce_add_sync(0xFFFFFFFFu, c);
     if (lane == src) count = c;
   }
   if (i < g.n) {
-    if (bins) {
+    if constexpr (BINS) {
       masks.lo[r] = mask.x;
       masks.hi[r] = mask.y;
-      masks.box[r] = tall || x1 - x0 >= 8 ? kLargeBox : ((uint32_t)y0 << 16 | (uint32_t)x0);
+      masks.box[r] = tall ? kLargeBox : ((uint32_t)y0 << 16 | (uint32_t)x0);
       masks.zbits[r] = __float_as_uint(z);
     } else {
       depth_key[r] = count ? __float_as_uint(z) : 0xFFFFFFFFu;
@@ -982,9 +1026,9 @@ void launch_project(const ngs_gaussians& g, const ViewParams* views, const CamPa
   if (g.n == 0) return;
   unsigned blocks = (unsigned)((g.n + 255) / 256) * rp.n_views;
   bool vec = ((uintptr_t)g.sh & 15) == 0;
-#define NGS_PROJECT(D, V) \
-  launch_pdl(project_kernel<D, V>, blocks, 256, 0, s, g, views, cam0, rp, rec, depth_key, tile_count, order, bins, \
-             masks)
+#define NGS_PROJECT(D, V)                                                                                            \
+  launch_pdl(bins ? project_kernel<D, V, true> : project_kernel<D, V, false>, blocks, 256, 0, s, g, views, cam0, rp, rec, \
+             depth_key, tile_count, order, bins, masks)
   switch (rp.sh_degree) {
     case 0: NGS_PROJECT(0, false); break;
     case 1:

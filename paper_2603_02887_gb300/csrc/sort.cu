@@ -421,7 +421,9 @@ constexpr int kWarpList = 256;     // longest list sorted by one warp
 constexpr int kWarpBuckets = 256;  // its buckets
 constexpr int kCtaList = kWarpList * (kSortThreads / 32);  // keys a CTA holds in shared memory
 constexpr int kCtaBuckets = kWarpBuckets * (kSortThreads / 32);
-constexpr uint32_t kHeavy = 48;  // a bucket with more keys is sorted by the network, not by counting
+// With more keys in one bucket, a list is sorted by the network, not by comparing each key with its bucket's: the
+// network of a CTA is 66 steps with a barrier each, so that it pays later.
+constexpr uint32_t kHeavy = 48, kHeavyCta = 160;
 
 // ranges[t].y holds tile t's count; afterwards ranges[t] = (o, o) with o the number of pairs in the tiles
 // before t of its block of kBinBlock tiles. `bases` receives the blocks' first pairs, *total the pair count:
@@ -729,24 +731,44 @@ __device__ __forceinline__ void cta_sort_list(const unsigned long long* __restri
   for (int j = 0; j < kPer; ++j)
     if (j * kSortThreads + tid < n) s_key[atomicAdd(&s_cnt[bucket(k[j], kCtaBuckets)], 1u)] = k[j];
   __syncthreads();
-  cta_write_run(s_key, s_cnt, n, 0, bucket, most > kHeavy, out);
+  cta_write_run(s_key, s_cnt, n, 0, bucket, most > kHeavyCta, out);
 }
 
-// A list of any length: taken in runs of consecutive buckets that shared memory holds, one reading of the list per
-// run. A bucket that alone exceeds it leaves the list to the network, in place in global memory.
+// Calls f(index, key) for every key, eight loads of a thread on their way at a time.
+template <typename F>
+__device__ __forceinline__ void for_keys(const unsigned long long* __restrict__ keys, uint32_t n, F f) {
+  constexpr int kFlight = 8;
+  for (uint32_t i0 = 0; i0 < n; i0 += kFlight * kSortThreads) {
+    unsigned long long k[kFlight];
+#pragma unroll
+    for (int j = 0; j < kFlight; ++j) {
+      const uint32_t i = i0 + j * kSortThreads + threadIdx.x;
+      k[j] = i < n ? keys[i] : 0ull;
+    }
+#pragma unroll
+    for (int j = 0; j < kFlight; ++j) {
+      const uint32_t i = i0 + j * kSortThreads + threadIdx.x;
+      if (i < n) f(i, k[j]);
+    }
+  }
+}
+
+// A list of any length: the keys' places by bucket go to `tmp` (n words), and runs of consecutive buckets that shared
+// memory holds are then sorted one after another. A bucket that alone exceeds it leaves the list to the network, in
+// place in global memory.
 __device__ __noinline__ void cta_sort_long_list(unsigned long long* keys, uint32_t n, uint32_t* __restrict__ out,
-                                                unsigned long long* s_key, uint32_t* s_cnt, uint32_t* s_red) {
+                                                uint32_t* tmp, unsigned long long* s_key, uint32_t* s_cnt,
+                                                uint32_t* s_red) {
   const uint32_t full = 0xFFFFFFFFu, tid = threadIdx.x;
   uint32_t hmin = full, hmax = 0, lmin = full, lmax = 0;
-  for (uint32_t i = tid; i < n; i += kSortThreads) {
-    const unsigned long long k = keys[i];
+  for_keys(keys, n, [&](uint32_t, unsigned long long k) {
     hmin = min(hmin, (uint32_t)(k >> 32));
     hmax = max(hmax, (uint32_t)(k >> 32));
     lmin = min(lmin, (uint32_t)k);
     lmax = max(lmax, (uint32_t)k);
-  }
+  });
   const BucketMap bucket = cta_bucket_map(hmin, hmax, lmin, lmax, s_cnt, s_red);
-  for (uint32_t i = tid; i < n; i += kSortThreads) atomicAdd(&s_cnt[bucket(keys[i], kCtaBuckets)], 1u);
+  for_keys(keys, n, [&](uint32_t, unsigned long long k) { atomicAdd(&s_cnt[bucket(k, kCtaBuckets)], 1u); });
   __syncthreads();
   const uint32_t most = cta_scan_buckets(s_cnt, s_red);
   if (most > (uint32_t)kCtaList) {
@@ -754,30 +776,36 @@ __device__ __noinline__ void cta_sort_long_list(unsigned long long* keys, uint32
     for (uint32_t i = tid; i < n; i += kSortThreads) out[i] = (uint32_t)keys[i];
     return;
   }
+  for_keys(keys, n,
+           [&](uint32_t i, unsigned long long k) { tmp[atomicAdd(&s_cnt[bucket(k, kCtaBuckets)], 1u)] = i; });
+  __syncthreads();  // s_cnt[b] is now the end of bucket b
   for (uint32_t b0 = 0, first = 0; first < n;) {
-    // buckets [b0, b1) hold at most kCtaList keys, list positions [first, last)
-    uint32_t b1 = kCtaBuckets, last = n;
-    if (n - first > (uint32_t)kCtaList) {
-      uint32_t l = b0 + 1, h = kCtaBuckets - 1;  // start(b0 + 1) - first <= kCtaList: no bucket is larger
-      while (l < h) {
-        const uint32_t mid = (l + h + 1) >> 1;
-        if (s_cnt[mid] - first <= (uint32_t)kCtaList) l = mid;
-        else h = mid - 1;
+    // buckets [b0, l] hold at most kCtaList keys, list positions [first, first + m): no bucket is larger
+    uint32_t l = b0, h = kCtaBuckets - 1;
+    while (l < h) {
+      const uint32_t mid = (l + h + 1) >> 1;
+      if (s_cnt[mid] - first <= (uint32_t)kCtaList) l = mid;
+      else h = mid - 1;
+    }
+    const uint32_t m = s_cnt[l] - first;
+    for (uint32_t i0 = 0; i0 < m; i0 += 4 * kSortThreads) {
+      uint32_t at[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t i = i0 + j * kSortThreads + tid;
+        at[j] = i < m ? tmp[first + i] : 0u;
       }
-      b1 = l;
-      last = s_cnt[b1];
-    }
-    __syncthreads();  // every thread has read the starts that the scatter advances to the ends
-    for (uint32_t i = tid; i < n; i += kSortThreads) {
-      const unsigned long long k = keys[i];
-      const uint32_t b = bucket(k, kCtaBuckets);
-      if (b >= b0 && b < b1) s_key[atomicAdd(&s_cnt[b], 1u) - first] = k;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t i = i0 + j * kSortThreads + tid;
+        if (i < m) s_key[i] = keys[at[j]];
+      }
     }
     __syncthreads();
-    cta_write_run(s_key, s_cnt, last - first, first, bucket, most > kHeavy, out);
+    cta_write_run(s_key, s_cnt, m, first, bucket, most > kHeavyCta, out);
     __syncthreads();
-    b0 = b1;
-    first = last;
+    b0 = l + 1;
+    first += m;
   }
 }
 
@@ -794,7 +822,7 @@ __device__ __forceinline__ uint2 tile_segment(const uint64_t* __restrict__ bases
 // its place in the work list of descending cost.
 __global__ void __launch_bounds__(kSortThreads, 5)
     tile_sort_kernel(unsigned long long* keys, uint32_t cap, const uint64_t* __restrict__ bases, uint32_t ntiles,
-                     const uint2* local, uint2* __restrict__ ranges, uint32_t* __restrict__ out, uint32_t big_ctas,
+                     const uint2* local, uint2* __restrict__ ranges, uint32_t* __restrict__ out, uint32_t* tmp, uint32_t big_ctas,
                      const uint32_t* __restrict__ big, uint32_t big_cap, const uint64_t* __restrict__ total,
                      uint32_t* __restrict__ sched, uint32_t* __restrict__ work) {
   pdl_wait();
@@ -816,7 +844,7 @@ __global__ void __launch_bounds__(kSortThreads, 5)
       if (l.y - l.x <= (uint32_t)kWarpList) continue;
       const uint2 r = tile_segment(bases, l, t, cap);
       const uint32_t n = r.y - r.x;
-      if (n > (uint32_t)kCtaList) cta_sort_long_list(keys + r.x, n, out + r.x, s_key, s_cnt, s_red);
+      if (n > (uint32_t)kCtaList) cta_sort_long_list(keys + r.x, n, out + r.x, tmp + r.x, s_key, s_cnt, s_red);
       else if (n) cta_sort_list(keys + r.x, n, out + r.x, s_key, s_cnt, s_red);
       __syncthreads();
       if (threadIdx.x == 0) finish(t, l, r);
@@ -912,13 +940,13 @@ void launch_tile_scan(uint2* ranges, uint32_t ntiles, uint64_t* bases, uint64_t*
 }
 
 void launch_tile_sort(uint64_t* keys, uint32_t cap, const uint64_t* bases, uint32_t ntiles, uint2* ranges, uint32_t* out,
-                      const uint32_t* big, uint32_t big_cap, const uint64_t* total, uint32_t* sched, uint32_t* work,
+                      uint32_t* tmp, const uint32_t* big, uint32_t big_cap, const uint64_t* total, uint32_t* sched, uint32_t* work,
                       int num_sms, cudaStream_t s) {
   constexpr uint32_t kTiles = kSortThreads / 32;
   const uint32_t big_ctas = std::min(ntiles, 4u * (uint32_t)std::max(num_sms, 1));  // one wave
   launch_pdl(tile_sort_kernel, big_ctas + (ntiles + kTiles - 1) / kTiles, kSortThreads, 0, s,
-             reinterpret_cast<unsigned long long*>(keys), cap, bases, ntiles, ranges, ranges, out, big_ctas, big, big_cap,
-             total, sched, work);
+             reinterpret_cast<unsigned long long*>(keys), cap, bases, ntiles, ranges, ranges, out, tmp, big_ctas, big,
+             big_cap, total, sched, work);
 }
 
 }  // namespace ngs

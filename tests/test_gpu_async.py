@@ -115,3 +115,26 @@ def test_status_without_render_is_an_error(rnd):
     with pytest.raises(_abi.NGSError):
         f.status()
     f.release()
+
+
+@pytest.mark.parametrize("graphs", [False, True])
+def test_synchronous_render_that_outgrows_its_frame(rnd, graphs):
+    """A frame's second and later synchronous renders are enqueued for what its pair buffers hold before the host has
+    the count: a render that does not fit, and one that again does, are exact, with the exact pair count."""
+    small, big = upload(synth.tiny_scene(3)), upload(synth.clustered_scene(30000, seed=22, sh_degree=3))
+    cam = synth.outside_camera(240, 160, 12.0)
+    rnd.set_graphs(graphs)
+    try:
+        want = {}
+        for name, params in (("small", small), ("big", big)):
+            img, od, f = rnd.render(params, cam, "lin", frame=Frame(rnd))
+            want[name] = (img.cpu().numpy(), od.cpu().numpy(), f.view()["n_pairs"])
+            f.release()
+        f = Frame(rnd)
+        for name in ("small", "big", "big", "small", "big"):
+            img, od, f = rnd.render(small if name == "small" else big, cam, "lin", frame=f)
+            assert f.status() == want[name][2]
+            assert np.array_equal(img.cpu().numpy(), want[name][0]) and np.array_equal(od.cpu().numpy(), want[name][1])
+        f.release()
+    finally:
+        rnd.set_graphs(False)
