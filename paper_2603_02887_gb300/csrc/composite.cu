@@ -126,10 +126,10 @@ __device__ __forceinline__ uint32_t next_tile(const uint32_t* __restrict__ work,
 // Staging of one chunk for the packed (two pixels per thread) forward and replay: every per-splat operand
 // duplicated, so one 16-byte shared load gives the operand pairs {a, a, b, b} of two FP32x2 instructions.
 template <int CH>
-struct PairStageBuf {
-  float4 q0[CH];  // {-u, -u, -v, -v}
-  float4 q1[CH];  // {A', A', B', B'}
-  float4 q2[CH];  // {C', C', L, L}
+struct PairStageBuf {  // (q0..q2 have an entry that is read ahead but never used)
+  float4 q0[CH + 1];  // {-u, -u, -v, -v}
+  float4 q1[CH + 1];  // {A', A', B', B'}
+  float4 q2[CH + 1];  // {C', C', L, L}
   float4 q3[CH];  // {E0, E0, E1, E1}
   float4 q4[CH];  // {E2, E2, record index (bits), 0}: one 16-byte load gives E2 and the atomics' target
 };
@@ -137,7 +137,7 @@ struct PairStageBuf {
 // The packed form (exponential and quadratic models) is used while its staging (72 B per record) stays
 // within 40 KB of static shared memory.
 template <int KIND, int CH>
-constexpr bool kPairForm = (KIND == NGS_MODEL_EXP || KIND == NGS_MODEL_QUAD) && sizeof(PairStageBuf<CH>) <= 40960;
+constexpr bool kPairForm = (KIND == NGS_MODEL_EXP || KIND == NGS_MODEL_QUAD) && sizeof(PairStageBuf<CH>) <= 41216;
 
 template <int B, int CH>
 __device__ __forceinline__ void stage_chunk_pairs(const float4* __restrict__ rec, const uint32_t* __restrict__ ids,
@@ -344,7 +344,7 @@ __device__ __forceinline__ void forward_tile(const float4* __restrict__ rec, con
 // each entry together in FP32x2 instructions. Each lane rounds exactly like the one-pixel form above, so
 // the image, the stop index and the replay state are the same bits. A pixel that has stopped, or that
 // does not composite the entry, gets alpha = 0, which leaves its sums exactly unchanged.
-template <int TW, int TH, int KIND, int CH>
+template <int TW, int TH, int KIND, int CH, bool AHEAD>
 __device__ __forceinline__ void forward_tile_pairs(const float4* __restrict__ rec, const uint32_t* __restrict__ ids,
                                                    const uint2* __restrict__ ranges, const RenderParams& rp,
                                                    const ViewParams* __restrict__ views, float* __restrict__ image,
@@ -378,14 +378,25 @@ __device__ __forceinline__ void forward_tile_pairs(const float4* __restrict__ re
     __syncthreads();
     const int cnt = (int)min((uint32_t)CH, range.y - base);
     if (__any_sync(kFull, !(done0 && done1))) {
-      for (int j = 0; j < cnt; ++j) {
+      auto exponent = [&](int j) {
         const float4 q0 = sb.q0[j], q1 = sb.q1[j], q2 = sb.q2[j];
         const float2 dx = __fadd2_rn(px, lo_hi(q0, false));
         const float2 adx = __fmul2_rn(lo_hi(q1, false), dx);
         const float2 dy = __fadd2_rn(py, lo_hi(q0, true));
         const float2 t = __ffma2_rn(lo_hi(q1, true), dy, adx);
         const float2 cdd = __fmul2_rn(__fmul2_rn(lo_hi(q2, false), dy), dy);
-        const float2 e = __fadd2_rn(lo_hi(q2, true), __ffma2_rn(dx, t, cdd));
+        return __fadd2_rn(lo_hi(q2, true), __ffma2_rn(dx, t, cdd));
+      };
+      float2 e_next;
+      if constexpr (AHEAD) e_next = exponent(0);
+      for (int j = 0; j < cnt; ++j) {
+        float2 e;
+        if constexpr (AHEAD) {  // the next entry's, while this one is composited
+          e = e_next;
+          e_next = exponent(j + 1);
+        } else {
+          e = exponent(j);
+        }
         const bool on0 = !done0 && e.x >= l2min, on1 = !done1 && e.y >= l2min;
         // warp-uniform: a lane that does not composite the entry (or has stopped) runs the step with
         // alpha = 0, which leaves its sums exactly as they were; the warp leaves the chunk once all of its
@@ -428,24 +439,33 @@ __device__ __forceinline__ void forward_tile_pairs(const float4* __restrict__ re
           c0 = on0;
           c1 = on1;
         } else {
-          // stop before the splat that would take T below t_eps
-          const float2 testT = __fmul2_rn(T, __ffma2_rn(alpha, neg, one));
-          const bool st0 = on0 && testT.x < rp.t_eps, st1 = on1 && testT.y < rp.t_eps;
-          if (st0) {
-            done0 = true;
-            stop0 = pos;
+          // stop before the splat that would take T below t_eps (only a pixel that composites can; it happens at most
+          // once per pixel, so the warp tests for it together)
+          float2 testT = __fmul2_rn(T, __ffma2_rn(alpha, neg, one)), a = alpha;
+          c0 = on0;
+          c1 = on1;
+          const bool st0 = testT.x < rp.t_eps, st1 = testT.y < rp.t_eps;
+          if (__any_sync(kFull, st0 || st1)) {
+            if (st0) {
+              done0 = true;
+              stop0 = pos;
+              c0 = false;
+              a.x = 0.f;
+              testT.x = T.x;
+            }
+            if (st1) {
+              done1 = true;
+              stop1 = pos;
+              c1 = false;
+              a.y = 0.f;
+              testT.y = T.y;
+            }
           }
-          if (st1) {
-            done1 = true;
-            stop1 = pos;
-          }
-          c0 = on0 && !st0;
-          c1 = on1 && !st1;
-          const float2 w = __fmul2_rn(make_float2(c0 ? alpha.x : 0.f, c1 ? alpha.y : 0.f), T);
+          const float2 w = __fmul2_rn(a, T);
           C0 = __ffma2_rn(E0, w, C0);
           C1 = __ffma2_rn(E1, w, C1);
           C2 = __ffma2_rn(E2, w, C2);
-          T = make_float2(c0 ? testT.x : T.x, c1 ? testT.y : T.y);
+          T = testT;
         }
         od0 += c0;
         od1 += c1;
@@ -502,7 +522,14 @@ constexpr int kFwdThreads = TW * TH / (kPairFwd<TW, TH, KIND, CH> ? 2 : 1);
 template <int TW, int TH, int KIND, int CH>
 constexpr int kFwdMinBlocks = (kPairFwd<TW, TH, KIND, CH> && KIND == NGS_MODEL_QUAD && TW * TH == 256) ? 9 : 1;
 
-template <int TW, int TH, int KIND, int CH, bool PERSIST>
+// How a launch walks the tiles: one CTA per tile; persistent CTAs over the work list; or one CTA per tile that reads
+// ahead, for frames of so few tiles that each warp's own latency is the time. Reading ahead takes the next entry's
+// exponent off the chain of dependent instructions of an entry, at the price of a few more instructions (1k Gaussians,
+// 128x128, exponential: 24.9 + 29.0 -> 22.6 + 26.9 us; 50k, 640x360, c = +0.5: 63 + 45 -> 56 + 42; but 500k, 1920x1080,
+// exponential: 187 + 349 -> 195 + 365).
+enum Walk { kTiles, kPersistent, kAhead };
+
+template <int TW, int TH, int KIND, int CH, Walk WALK>
 __global__ void __launch_bounds__(kFwdThreads<TW, TH, KIND, CH>, kFwdMinBlocks<TW, TH, KIND, CH>)
     composite_forward_kernel(const float4* __restrict__ rec,
                                                                    const uint32_t* __restrict__ ids,
@@ -518,11 +545,11 @@ __global__ void __launch_bounds__(kFwdThreads<TW, TH, KIND, CH>, kFwdMinBlocks<T
   __shared__ Buf sb;
   auto one_tile = [&](uint32_t tile) {
     if constexpr (kPairFwd<TW, TH, KIND, CH>)
-      forward_tile_pairs<TW, TH, KIND, CH>(rec, ids, ranges, rp, views, image, overdraw, state, tile, sb);
+      forward_tile_pairs<TW, TH, KIND, CH, WALK == kAhead>(rec, ids, ranges, rp, views, image, overdraw, state, tile, sb);
     else
       forward_tile<TW, TH, KIND, CH>(rec, ids, ranges, rp, views, image, overdraw, state, tile, sb);
   };
-  if constexpr (PERSIST) {
+  if constexpr (WALK == kPersistent) {
     __shared__ uint32_t s_next;
     for (;;) {
       const uint32_t tile = next_tile(work, counter, rp.n_tiles, &s_next);
@@ -766,7 +793,7 @@ __device__ __forceinline__ void bwd_pair_step(BwdPair& p, float2 e, float2 dx, f
   v[8] = c2.x + c2.y;
 }
 
-template <int TW, int TH, int KIND, int CH>
+template <int TW, int TH, int KIND, int CH, bool AHEAD>
 __device__ __forceinline__ void backward_tile_pairs(const float4* __restrict__ rec, const uint32_t* __restrict__ ids,
                                                     const uint2* __restrict__ ranges, const RenderParams& rp,
                                                     const ViewParams* __restrict__ views,
@@ -831,9 +858,18 @@ __device__ __forceinline__ void backward_tile_pairs(const float4* __restrict__ r
     __syncthreads();
     if (base < warp_last) {
       const int cnt = (int)(min(warp_last, min(base + (uint32_t)CH, range.y)) - base);
+      float2 dx_next, dy_next, e_next;
+      if constexpr (AHEAD) e_next = pair_log2_alpha(p, sb.q0[0], sb.q1[0], sb.q2[0], dx_next, dy_next);
       for (int j = 0; j < cnt; ++j) {
-        float2 dx, dy;
-        const float2 e = pair_log2_alpha(p, sb.q0[j], sb.q1[j], sb.q2[j], dx, dy);
+        float2 dx, dy, e;
+        if constexpr (AHEAD) {  // the next entry's, while this one is differentiated
+          dx = dx_next;
+          dy = dy_next;
+          e = e_next;
+          e_next = pair_log2_alpha(p, sb.q0[j + 1], sb.q1[j + 1], sb.q2[j + 1], dx_next, dy_next);
+        } else {
+          e = pair_log2_alpha(p, sb.q0[j], sb.q1[j], sb.q2[j], dx, dy);
+        }
         const uint32_t pos = base + j;
         const bool on0 = pos < p.last0 && e.x >= rp.log2_alpha_min;
         const bool on1 = pos < p.last1 && e.y >= rp.log2_alpha_min;
@@ -963,7 +999,7 @@ __device__ __forceinline__ void backward_tile(const float4* __restrict__ rec, co
   }
 }
 
-template <int TW, int TH, int KIND, int CH, bool PERSIST>
+template <int TW, int TH, int KIND, int CH, Walk WALK>
 __global__ void __launch_bounds__(TW* TH / kBwdPix) composite_backward_kernel(const float4* __restrict__ rec,
                                                                         const uint32_t* __restrict__ ids,
                                                                         const uint2* __restrict__ ranges,
@@ -980,11 +1016,11 @@ __global__ void __launch_bounds__(TW* TH / kBwdPix) composite_backward_kernel(co
   __shared__ uint32_t s_id[kPairForm<KIND, CH> ? 1 : CH];  // the packed form carries the index in its q4
   auto one_tile = [&](uint32_t tile) {
     if constexpr (kPairForm<KIND, CH>)
-      backward_tile_pairs<TW, TH, KIND, CH>(rec, ids, ranges, rp, views, dl_dimage, state, grad2d, tile, sb);
+      backward_tile_pairs<TW, TH, KIND, CH, WALK == kAhead>(rec, ids, ranges, rp, views, dl_dimage, state, grad2d, tile, sb);
     else
       backward_tile<TW, TH, KIND, CH>(rec, ids, ranges, rp, views, dl_dimage, state, grad2d, tile, sb, s_id);
   };
-  if constexpr (PERSIST) {
+  if constexpr (WALK == kPersistent) {
     __shared__ uint32_t s_next;
     for (;;) {
       const uint32_t tile = next_tile(work, counter, rp.n_tiles, &s_next);
@@ -1008,10 +1044,15 @@ struct Launch {
 // One CTA per tile, or one wave of persistent CTAs (SM count x resident CTAs per SM).
 template <typename Kernel>
 static unsigned grid_for(Kernel k, int threads, const Launch& L, uint32_t n_tiles) {
-  if (!L.counter) return n_tiles;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
   return (unsigned)std::min<uint64_t>((uint64_t)per_sm * (uint64_t)L.num_sms, n_tiles);
+}
+
+// Few tiles: at most 32 warps per SM in all (one 8 x 8 pixel block per warp).
+template <int TW, int TH>
+static bool few_tiles(const Launch& L, uint32_t n_tiles) {
+  return (uint64_t)n_tiles * (TW * TH / 64) <= 32ull * (uint64_t)std::max(L.num_sms, 1);
 }
 
 template <int TW, int TH, int KIND, int CH>
@@ -1019,9 +1060,15 @@ void forward_launch(const float4* rec, const uint32_t* ids, const uint2* ranges,
                     const ViewParams* views, float* image, int32_t* overdraw, float4* state, const Launch& L,
                     cudaStream_t s) {
   constexpr int threads = kFwdThreads<TW, TH, KIND, CH>;
-  auto k = L.counter ? composite_forward_kernel<TW, TH, KIND, CH, true> : composite_forward_kernel<TW, TH, KIND, CH, false>;
-  launch_pdl(k, grid_for(k, threads, L, rp.n_tiles), threads, 0, s, rec, ids, ranges, rp, views, image, overdraw, state,
-             L.work, L.counter);
+  auto k = composite_forward_kernel<TW, TH, KIND, CH, kTiles>;
+  unsigned grid = rp.n_tiles;
+  if (kPairFwd<TW, TH, KIND, CH> && few_tiles<TW, TH>(L, rp.n_tiles)) {
+    k = composite_forward_kernel<TW, TH, KIND, CH, kPairFwd<TW, TH, KIND, CH> ? kAhead : kTiles>;
+  } else if (L.counter) {
+    k = composite_forward_kernel<TW, TH, KIND, CH, kPersistent>;
+    grid = grid_for(k, threads, L, rp.n_tiles);
+  }
+  launch_pdl(k, grid, threads, 0, s, rec, ids, ranges, rp, views, image, overdraw, state, L.work, L.counter);
 }
 
 template <int TW, int TH, int KIND, int CH>
@@ -1029,10 +1076,15 @@ void backward_launch(const float4* rec, const uint32_t* ids, const uint2* ranges
                      const ViewParams* views, const float* dl, const float4* state, float4* grad2d, const Launch& L,
                      cudaStream_t s) {
   constexpr int threads = TileGeom<TW, TH, kBwdPix>::kThreads;
-  auto k =
-      L.counter ? composite_backward_kernel<TW, TH, KIND, CH, true> : composite_backward_kernel<TW, TH, KIND, CH, false>;
-  launch_pdl(k, grid_for(k, threads, L, rp.n_tiles), threads, 0, s, rec, ids, ranges, rp, views, dl, state, grad2d,
-             L.work, L.counter);
+  auto k = composite_backward_kernel<TW, TH, KIND, CH, kTiles>;
+  unsigned grid = rp.n_tiles;
+  if (kPairForm<KIND, CH> && few_tiles<TW, TH>(L, rp.n_tiles)) {
+    k = composite_backward_kernel<TW, TH, KIND, CH, kPairForm<KIND, CH> ? kAhead : kTiles>;
+  } else if (L.counter) {
+    k = composite_backward_kernel<TW, TH, KIND, CH, kPersistent>;
+    grid = grid_for(k, threads, L, rp.n_tiles);
+  }
+  launch_pdl(k, grid, threads, 0, s, rec, ids, ranges, rp, views, dl, state, grad2d, L.work, L.counter);
 }
 
 template <int TW, int TH, int KIND>

@@ -265,3 +265,32 @@ def test_autotune_returns_a_valid_fastest_configuration(rnd, clustered):
     a = rnd.render_batch(params, cams, "sup")
     b = rnd.render_batch(params, cams, "sup", options=best)
     assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("model", MODELS + ["blend", "vicini"])
+@pytest.mark.parametrize("tile", [(8, 8), (16, 16)])
+def test_small_frames_walk_the_lists_alike(rnd, clustered, model, tile):
+    """Frames of few tiles read ahead, larger ones do not: a batch of many views of a size that alone is small equals
+    the single renders bit for bit, image, overdraw and replay state; the gradients agree up to the order of sums."""
+    scene, _ = clustered
+    params = upload(scene)
+    views = 30 if tile == (8, 8) else 40  # x 384 or 96 tiles, more than 32 warps per SM
+    cams = synth.orbit_cameras(views, radius=12.0, seed=11, resolutions=((190, 124),))
+    opts = dict(tile_w=tile[0], tile_h=tile[1])
+    images, overdraw, frame = rnd.render_batch(params, cams, model, options=opts)
+    state = batch_arrays(frame)["state"]
+    dl = torch.ones_like(images)
+    grads = {k: v.clone() for k, v in rnd.backward(frame, params, dl).items()}
+    total = {k: torch.zeros_like(v, dtype=torch.float64) for k, v in grads.items()}
+    size = 190 * 124
+    for v, cam in enumerate(cams):
+        img, od, f = rnd.render(params, cam, model, options=opts)
+        assert torch.equal(images[v * size:(v + 1) * size].view_as(img), img), v
+        assert torch.equal(overdraw[v * size:(v + 1) * size].view_as(od), od), v
+        if v % 10 == 0:
+            assert np.array_equal(_bits(state[v * size:(v + 1) * size]), _bits(frame_arrays(f)["state"].reshape(-1, 8)))
+        for k, g in rnd.backward(f, params, torch.ones_like(img)).items():
+            total[k] += g.double()
+        rnd.recycle(f)
+    for k, g in grads.items():  # FP32 sums of up to 30 views in another order
+        assert torch.allclose(g.double(), total[k], rtol=1e-4, atol=1e-5 * float(total[k].abs().max())), k
