@@ -870,6 +870,20 @@ __device__ __forceinline__ void add_view_gradient(const RawParams& prm, const Ca
       gsh[3 * k + 2] = d2 * st.Y[k];
     }
     store_sh<K, VEC>(dsh_dst, gsh);
+  } else if (dsh_dst) {  // the views' sum stands in shared memory
+    if constexpr (VEC) {
+      const float d[3] = {d0, d1, d2};
+      float4* const sum = reinterpret_cast<float4*>(dsh_dst);
+#pragma unroll
+      for (int q = 0; q < 3 * K / 4; ++q) {
+        float4 t = sum[q];
+        t.x += d[(4 * q) % 3] * st.Y[(4 * q) / 3];
+        t.y += d[(4 * q + 1) % 3] * st.Y[(4 * q + 1) / 3];
+        t.z += d[(4 * q + 2) % 3] * st.Y[(4 * q + 2) / 3];
+        t.w += d[(4 * q + 3) % 3] * st.Y[(4 * q + 3) / 3];
+        sum[q] = t;
+      }
+    }
   } else {
 #pragma unroll
     for (int k = 0; k < K; ++k) {
@@ -903,19 +917,28 @@ __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefe
 // The CTAs stride over blocks of 128 Gaussians (a grid of one wave for a single view): while a block
 // computes, the next block's lines are already on their way into L2, so that DRAM stays busy through the
 // long arithmetic stretch of each block.
+// A batch with 16-byte SH rows keeps both the coefficients and the views' SH gradient sums in shared memory (CTAs of 64,
+// six per SM at 168 registers): in registers they took 250, which left 8 warps per SM to hide the chain's latency
+// (32 % of issue slots used). 32 views of 3M Gaussians, 8 x 8 tiles: 6.36 -> 4.98 ms, 4 views of 500k 184 -> 152 us. Eight CTAs
+// (128 registers) spill inside the chain and take 8.57 ms, five 5.10 ms.
+template <bool VEC, bool MULTI>
+constexpr int kBackThreads = VEC && MULTI ? 64 : 128;
 template <int DEG, bool VEC, bool MULTI>
-__global__ void __launch_bounds__(128, MULTI ? 1 : 4) project_backward_kernel(ngs_gaussians g, const ViewParams* __restrict__ views,
+__global__ void __launch_bounds__(kBackThreads<VEC, MULTI>, MULTI ? (VEC ? 6 : 1) : 4) project_backward_kernel(ngs_gaussians g, const ViewParams* __restrict__ views,
                                                                CamParams cam0, RenderParams rp,
                                                                const uint32_t* tile_count, const float4* grad2d,
                                                                ngs_grads out) {
   pdl_wait();
   constexpr int K = (DEG + 1) * (DEG + 1);
-  // One view with 16-byte SH rows: each warp moves its 32 Gaussians' SH blocks (contiguous in memory)
+  // 16-byte SH rows: each warp moves its 32 Gaussians' SH blocks (contiguous in memory)
   // between global and shared memory with coalesced 16-byte accesses; each thread then reads its
   // coefficients and writes its SH gradient there (row stride Q + 1 float4 against bank conflicts).
-  constexpr bool kStage = VEC && !MULTI;
+  constexpr bool kStage = VEC;
+  constexpr int kThreads = kBackThreads<VEC, MULTI>;
   constexpr int Q = VEC ? 3 * K / 4 : 1;  // float4 per Gaussian
-  __shared__ float4 s_sh[kStage ? 128 * (Q + 1) : 1];
+  __shared__ float4 s_sh[kStage ? kThreads * (Q + 1) : 1];
+  __shared__ float4 s_sum[kStage && MULTI ? kThreads * (Q + 1) : 1];  // a batch's SH gradients
+  float4* const s_out = MULTI ? s_sum : s_sh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   for (int64_t b0 = (int64_t)blockIdx.x * blockDim.x; b0 < g.n; b0 += step) {
@@ -985,12 +1008,29 @@ __global__ void __launch_bounds__(128, MULTI ? 1 : 4) project_backward_kernel(ng
         }
       } else {
         const RawParams prm = load_params(g, i);
-        for (int v = 0; v < (int)rp.n_views; ++v) {
+        const float* sh_src = g.sh + (int64_t)i * K * 3;
+        float* sum = nullptr;
+        if constexpr (kStage) {
+          sh_src = reinterpret_cast<const float*>(my_sh);
+          sum = reinterpret_cast<float*>(&s_sum[threadIdx.x * (Q + 1)]);
+          store_sh<K, VEC>(sum, acc.sh);
+        }
+        // the counts are read two views ahead, the record gradients requested one view ahead
+        const int views_n = (int)rp.n_views;
+        uint32_t here = tile_count[i], next = views_n > 1 ? tile_count[(int64_t)g.n + i] : 0u;
+        for (int v = 0; v < views_n; ++v) {
           const int64_t r = (int64_t)v * g.n + i;
-          if (tile_count[r] == 0) continue;
+          const uint32_t count = here;
+          here = next;
+          if (here != 0) {
+            prefetch_l1(grad2d + 3 * (r + g.n));
+            prefetch_l1(grad2d + 3 * (r + g.n) + 2);
+          }
+          next = v + 2 < views_n ? tile_count[r + 2 * (int64_t)g.n] : 0u;
+          if (count == 0) continue;
           const CamParams cam = views[v].cam;
           add_view_gradient<DEG, VEC, false>(prm, cam, rp, i, grad2d[3 * r], grad2d[3 * r + 1], grad2d[3 * r + 2],
-                                             acc, out, g.sh + (int64_t)i * K * 3, nullptr);
+                                             acc, out, sh_src, sum);
         }
       }
       if (!written) {  // the sums over views (or zeros: culled in every view)
@@ -1002,8 +1042,8 @@ __global__ void __launch_bounds__(128, MULTI ? 1 : 4) project_backward_kernel(ng
 #pragma unroll
         for (int k = 0; k < 4; ++k) out.d_quats[4 * (int64_t)i + k] = acc.q[k];
         out.d_opacity_logits[i] = acc.op;
-        if constexpr (kStage) store_sh<K, VEC>(reinterpret_cast<float*>(my_sh), acc.sh);
-        else store_sh<K, VEC>(out.d_sh + (int64_t)i * K * 3, acc.sh);
+        if constexpr (!kStage) store_sh<K, VEC>(out.d_sh + (int64_t)i * K * 3, acc.sh);
+        else if constexpr (!MULTI) store_sh<K, VEC>(reinterpret_cast<float*>(my_sh), acc.sh);
       }
     }
     if constexpr (kStage) {
@@ -1011,7 +1051,7 @@ __global__ void __launch_bounds__(128, MULTI ? 1 : 4) project_backward_kernel(ng
       float4* dst = reinterpret_cast<float4*>(out.d_sh) + g0 * Q;
       for (int idx = lane; idx < warp_n * Q; idx += 32) {
         const int j = idx / Q;
-        dst[idx] = s_sh[(warp * 32 + j) * (Q + 1) + (idx - j * Q)];
+        dst[idx] = s_out[(warp * 32 + j) * (Q + 1) + (idx - j * Q)];
       }
       __syncwarp();  // the next block's staging overwrites these rows
     }
@@ -1065,7 +1105,8 @@ static void project_backward_views(const ngs_gaussians& g, const ViewParams* vie
                                    const ngs_grads& out, int num_sms, cudaStream_t s) {
   const int64_t blocks = (g.n + 127) / 128;
   if (rp.n_views > 1) {
-    launch_pdl(project_backward_kernel<DEG, VEC, true>, (unsigned)blocks, 128, 0, s, g, views, cam0, rp, tile_count,
+    constexpr int threads = kBackThreads<VEC, true>;
+    launch_pdl(project_backward_kernel<DEG, VEC, true>, (unsigned)((g.n + threads - 1) / threads), threads, 0, s, g, views, cam0, rp, tile_count,
                grad2d, out);
   } else {
     // one wave: 4 CTAs per SM (the kernel's register bound)

@@ -294,3 +294,36 @@ def test_small_frames_walk_the_lists_alike(rnd, clustered, model, tile):
         rnd.recycle(f)
     for k, g in grads.items():  # FP32 sums of up to 30 views in another order
         assert torch.allclose(g.double(), total[k], rtol=1e-4, atol=1e-5 * float(total[k].abs().max())), k
+
+
+@pytest.mark.parametrize("degree", [0, 1, 2, 3])
+@pytest.mark.parametrize("n", [1, 31, 64, 65, 200])
+def test_batch_parameter_gradients_are_the_views_sums(rnd, n, degree):
+    """The projection's adjoint over a batch: block remainders, every SH degree, rows on 16-byte boundaries and not, and
+    views that see some or all of the Gaussians."""
+    scene = synth.clustered_scene(n, seed=n + degree, sh_degree=degree)
+    cams = [synth.outside_camera(64, 48, 12.0), synth.outside_camera(33, 70, 9.0)]
+    cams += [synth.outside_camera(40, 40, 0.5), synth.outside_camera(50, 31, 20.0)]  # the first inside the cloud
+    for shift in (0, 1):
+        params = upload(scene)
+        store = torch.empty(params["sh"].numel() + 4, device="cuda")
+        sh = store[shift:shift + params["sh"].numel()].view_as(params["sh"])
+        sh.copy_(params["sh"])
+        params["sh"] = sh
+        images, _, frame = rnd.render_batch(params, cams, "lin")
+        gen = torch.Generator(device="cuda").manual_seed(3)
+        dl = torch.randn(images.shape, generator=gen, device="cuda")
+        grads = {k: v.clone() for k, v in rnd.backward(frame, params, dl).items()}
+        rnd.recycle(frame)
+        total, scale, at = {}, {}, 0
+        for cam in cams:
+            size = cam["width"] * cam["height"]
+            img, _, f = rnd.render(params, cam, "lin")
+            one = rnd.backward(f, params, dl[at:at + size].view_as(img).contiguous())
+            for k, g in one.items():
+                total[k] = total.get(k, 0) + g.double()
+                scale[k] = max(scale.get(k, 0.0), float(g.abs().max()))
+            at += size
+            rnd.recycle(f)
+        for k, g in grads.items():  # FP32 sums of four views and of their pixels in another order
+            assert torch.allclose(g.double(), total[k].view_as(g), rtol=1e-4, atol=1e-5 * scale[k] + 1e-12), k
