@@ -281,8 +281,11 @@ static size_t pair_keys_bytes(const BufferPlan& b) { return 2 * fresh_bytes(b.pa
 static size_t plan_frame_pairs(const BufferPlan& b) { return pair_keys_bytes(b) + 2 * fresh_bytes(b.pair_val); }
 
 // Which of the two ways builds the tile lists: counting (per-tile segments sorted on their own) or the global
-// radix sorts.
-constexpr uint64_t kBinMaxRecordsPerTile = 1024;
+// radix sorts. Counting takes an atomic per pair on its tile's word, twice, and these serialise where few tiles take many
+// records; the radix sorts cost some 20 launches and 16 B per pair and pass. Projection to tile ranges in us, counting /
+// radix: 61 records per tile 136 / 204 (500k, 1920x1080), 217 91 / 123 (200k, 640x360), 285 49 / 87 (20k, 160x100),
+// 384 94 / 104 (100k, 320x200), 461 302 / 266 (1M, 900x600), 543 179 / 172 (500k, 640x360), 923 980 / 450 (2M, 900x600).
+constexpr uint64_t kBinMaxRecordsPerTile = 384;
 static bool use_bins(uint64_t R, uint64_t ntiles) { return R <= kBinMaxRecordsPerTile * ntiles; }
 static size_t plan_context(const BufferPlan& b) {
   return fresh_bytes(b.scan_tmp) + fresh_bytes(b.total) + grown_size(grown_size(0, b.hist1), b.hist2);

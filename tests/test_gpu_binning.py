@@ -47,3 +47,20 @@ def test_tile_lists_match_the_oracle(n, depths, schedule):
     assert np.array_equal(fa["values"], vals)
     assert np.array_equal(fa["ranges"].astype(np.int64), ranges)
     r.close()
+
+
+@pytest.mark.parametrize("n", [9000, 24576, 24577])  # 384 records per tile: the last counted, and the first radix-sorted, size
+@pytest.mark.parametrize("depths", ["all", "most", "9"])
+def test_long_lists_and_the_limit_of_counting(n, depths):
+    """Lists longer than a CTA's shared memory in a frame of 64 tiles, most of them empty."""
+    scene = _scene(n, depths, seed=n)
+    cam = synth.pinhole(np.concatenate([np.eye(3), np.zeros((3, 1))], 1), 128, 128, 80.0, 80.0)
+    r = Renderer("cuda:0")
+    img, od, frame = r.render(upload(scene), cam, "sup")
+    fa = frame_arrays(frame)
+    keys, vals, ranges = binning.sorted_pairs(fa["records"], fa["view"]["log2_alpha_min"], 16, 16, 128, 128)
+    assert int((ranges[:, 1] - ranges[:, 0]).max()) > 2048
+    assert np.array_equal(fa["keys"], keys)
+    assert np.array_equal(fa["values"], vals)
+    assert np.array_equal(fa["ranges"].astype(np.int64), ranges)
+    r.close()
