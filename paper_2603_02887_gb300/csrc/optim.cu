@@ -102,20 +102,111 @@ __global__ void accumulate_kernel(const float* __restrict__ d_means, int64_t n, 
   }
 }
 
-// decision per Gaussian: 0 prune, 1 keep, 2 split candidate
-__global__ void densify_decide_kernel(const float* __restrict__ logits, const float* __restrict__ log_scales,
-                                      const float* __restrict__ accum, const float* __restrict__ count, int64_t n,
-                                      ngs_densify_cfg cfg, uint32_t* __restrict__ decision,
-                                      uint32_t* __restrict__ is_split) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// ---- split / prune: one kernel decides and counts, one moves the rows -------------------------------------
+//
+// A Gaussian's place among the new ones is the number of survivors before it plus that of the granted splits before it,
+// and the granted ones are the first `allowed` candidates: so one scan of (survivors, candidates) gives every place
+// once the totals are known: two launches, where a scan for the candidates' ranks and one for the places took 13. A call for
+// 100k Gaussians of degree 3, the counts read back: 206 -> 135 us.
+
+constexpr int kPlanThreads = 256, kPlanBlock = 4 * kPlanThreads;
+// A Gaussian's plan word: the survivors (11 bits) and candidates (11 bits) before it in its block of kPlanBlock, and
+// its decision: 0 prune, 1 keep, 2 split candidate.
+constexpr uint32_t kPlanBits = 11, kPlanMask = (1u << kPlanBits) - 1u;
+static_assert(kPlanBlock <= (int)kPlanMask + 1, "the counts before an item of its block");
+
+struct DensifyTotals {
+  uint64_t blocks_done;  // zero before and after a launch
+  uint64_t allowed;      // granted splits
+};
+
+__device__ __forceinline__ uint32_t densify_decision(const float* __restrict__ logits, const float* __restrict__ log_scales,
+                                                     const float* __restrict__ accum, const float* __restrict__ count,
+                                                     int64_t i, const ngs_densify_cfg& cfg) {
   const float op = 1.f / (1.f + expf(-logits[i]));
   const float smax = expf(fmaxf(log_scales[3 * i], fmaxf(log_scales[3 * i + 1], log_scales[3 * i + 2])));
-  uint32_t d = 1;
-  if (cfg.prune && (op < cfg.min_opacity || smax < cfg.min_scale)) d = 0;
-  else if (cfg.split && count[i] > 0.f && accum[i] / count[i] > cfg.grad_threshold) d = 2;
-  decision[i] = d;
-  is_split[i] = d == 2 ? 1u : 0u;
+  if (cfg.prune && (op < cfg.min_opacity || smax < cfg.min_scale)) return 0;
+  return cfg.split && count[i] > 0.f && accum[i] / count[i] > cfg.grad_threshold ? 2 : 1;
+}
+
+// Inclusive prefix sum over the warp.
+template <typename T>
+__device__ __forceinline__ T warp_inclusive(T x) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const T y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+
+// Plan words, and bases[b] = (survivors | candidates << 32) before block b: the block that finishes last scans the blocks'
+// counts (no block waits on another), grants the splits and publishes the new number of Gaussians.
+__global__ void __launch_bounds__(kPlanThreads) densify_plan_kernel(const float* __restrict__ logits,
+                                                                    const float* __restrict__ log_scales,
+                                                                    const float* __restrict__ accum,
+                                                                    const float* __restrict__ count, int64_t n,
+                                                                    ngs_densify_cfg cfg, uint32_t* __restrict__ plan,
+                                                                    uint64_t* bases, DensifyTotals* totals,
+                                                                    uint64_t* mirror) {
+  pdl_wait();
+  __shared__ uint64_t s_warp[kPlanThreads / 32];
+  __shared__ bool s_last;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t i0 = (int64_t)blockIdx.x * kPlanBlock + 4 * tid;
+  uint32_t d[4], mine = 0;  // survivors | candidates << 16
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    d[k] = i0 + k < n ? densify_decision(logits, log_scales, accum, count, i0 + k, cfg) : 0u;
+    mine += (d[k] != 0 ? 1u : 0u) + (d[k] == 2 ? 1u << 16 : 0u);
+  }
+  const uint32_t incl = warp_inclusive(mine);
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  uint32_t run = incl - mine, all = 0;
+#pragma unroll
+  for (int w = 0; w < kPlanThreads / 32; ++w) {
+    if (w < warp) run += (uint32_t)s_warp[w];
+    all += (uint32_t)s_warp[w];
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (i0 + k < n) plan[i0 + k] = (run & 0xFFFFu) | (run >> 16) << kPlanBits | d[k] << (2 * kPlanBits);
+    run += (d[k] != 0 ? 1u : 0u) + (d[k] == 2 ? 1u << 16 : 0u);
+  }
+  if (tid == 0) {
+    bases[blockIdx.x] = (uint64_t)(all & 0xFFFFu) | (uint64_t)(all >> 16) << 32;
+    __threadfence();
+    s_last = atomicAdd(reinterpret_cast<unsigned long long*>(&totals->blocks_done), 1ull) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  uint64_t carry = 0;  // both counts stay below 2^30
+  for (uint32_t b = 0; b < gridDim.x; b += kPlanThreads) {
+    const uint32_t at = b + tid;
+    const uint64_t v = at < gridDim.x ? __ldcg(reinterpret_cast<unsigned long long*>(bases) + at) : 0ull;
+    const uint64_t in = warp_inclusive(v);
+    __syncthreads();  // the previous use of s_warp is over
+    if (lane == 31) s_warp[warp] = in;
+    __syncthreads();
+    uint64_t before = carry + in - v;
+#pragma unroll
+    for (int w = 0; w < kPlanThreads / 32; ++w) {
+      if (w < warp) before += s_warp[w];
+      carry += s_warp[w];
+    }
+    if (at < gridDim.x) bases[at] = before;
+  }
+  if (tid == 0) {
+    const int64_t survivors = (int64_t)(carry & 0xFFFFFFFFu), candidates = (int64_t)(carry >> 32);
+    const int64_t room = cfg.max_gaussians > survivors ? cfg.max_gaussians - survivors : 0;
+    totals->allowed = (uint64_t)min(candidates, room);
+    totals->blocks_done = 0;
+    *mirror = (uint64_t)survivors + totals->allowed;
+    __threadfence_system();
+  }
 }
 
 __device__ __forceinline__ void quat_axis(const float* q, int a, float* r) {
@@ -139,94 +230,102 @@ __device__ __forceinline__ void quat_axis(const float* q, int a, float* r) {
 
 struct DensifyArgs {
   ParamPtrs src, src_m, src_v, dst, dst_m, dst_v;
-  int K3;  // 3 (sh_degree + 1)^2
+  bool vec[5];  // the array's six pointers are 16-byte aligned
+  int K3;       // 3 (sh_degree + 1)^2
 };
 
-__global__ void iota_kernel(uint32_t* __restrict__ out, int64_t n) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) out[i] = (uint32_t)i;
-}
-
-// splits allowed under the cap: min(candidates, max(0, cap - survivors)); survivors = n - pruned
-__global__ void densify_allowed_kernel(const uint64_t* __restrict__ cand_total,
-                                       const uint64_t* __restrict__ prune_total, int64_t n, int64_t cap,
-                                       uint32_t* __restrict__ allowed) {
-  const int64_t survivors = n - (int64_t)*prune_total;
-  const int64_t room = cap > survivors ? cap - survivors : 0;
-  *allowed = (uint32_t)min((int64_t)*cand_total, room);
-}
-
-// number of pruned Gaussians (decision 0), one atomic per warp
-__global__ void count_pruned_kernel(const uint32_t* __restrict__ decision, int64_t n, uint64_t* __restrict__ pruned) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const uint32_t b = __ballot_sync(0xFFFFFFFFu, i < n && decision[i] == 0);
-  if ((threadIdx.x & 31) == 0 && b) atomicAdd(reinterpret_cast<unsigned long long*>(pruned), (unsigned long long)__popc(b));
-}
-
-// output count per Gaussian: 0 pruned, 2 a granted split, else 1
-__global__ void densify_count_kernel(const uint32_t* __restrict__ decision, const uint32_t* __restrict__ rank,
-                                     const uint32_t* __restrict__ allowed, int64_t n, uint32_t* __restrict__ outc) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint32_t d = decision[i];
-  outc[i] = d == 0 ? 0u : (d == 2 && rank[i] < *allowed ? 2u : 1u);
-}
-
-// Array gi (W floats per Gaussian) of kApplyRows Gaussians from i0 on: a thread per float, so that reads and writes
-// are coalesced (a thread per Gaussian moved 59-float rows one float at a time: a split / prune of 100k Gaussians took
-// 310 us on GB300, 203 us so).
+// What becomes of each of a CTA's kApplyRows Gaussians: `copies` (0 pruned, 1 kept, 2 split) from row `to` on; a split's
+// longest axis, half its extent along it and its direction.
 constexpr int kApplyThreads = 256, kApplyRows = 64;
-template <int W>
-__device__ __forceinline__ void apply_array(const DensifyArgs& a, int gi, const uint32_t* __restrict__ outc,
-                                            const uint32_t* __restrict__ pos, int64_t i0, int64_t n) {
-  const int rows = (int)(n - i0 < kApplyRows ? n - i0 : kApplyRows);
-  for (int e = threadIdx.x; e < rows * W; e += kApplyThreads) {
-    const int r = e / W, k = e - r * W;
-    const int64_t i = i0 + r, from = i * W + k;
-    const uint32_t c = outc[i];
+struct ApplyRows {
+  uint32_t copies[kApplyRows], to[kApplyRows];
+  int axis[kApplyRows];
+  float half[kApplyRows], along[kApplyRows][3];
+};
+
+// Array gi (W floats per Gaussian, moved as VW at a time): a thread per element, so that reads and writes are coalesced.
+template <int W, typename V>
+__device__ __forceinline__ void apply_array(const DensifyArgs& a, int gi, const ApplyRows& rows, int64_t i0, int n_rows) {
+  constexpr int E = W / (int)(sizeof(V) / sizeof(float));  // elements of a row
+  const V *const src = reinterpret_cast<const V*>(a.src.p[gi]) + i0 * E;
+  const V *const src_m = reinterpret_cast<const V*>(a.src_m.p[gi]) + i0 * E;
+  const V *const src_v = reinterpret_cast<const V*>(a.src_v.p[gi]) + i0 * E;
+  V *const dst = reinterpret_cast<V*>(a.dst.p[gi]), *const dst_m = reinterpret_cast<V*>(a.dst_m.p[gi]);
+  V* const dst_v = reinterpret_cast<V*>(a.dst_v.p[gi]);
+  for (int e = threadIdx.x; e < n_rows * E; e += kApplyThreads) {
+    const int r = e / E, k = e - r * E;
+    const uint32_t c = rows.copies[r];
     if (c == 0) continue;
-    const int64_t to = (int64_t)pos[i] * W + k;
-    const float val = a.src.p[gi][from];
+    const int64_t to = (int64_t)rows.to[r] * E + k;
+    const V val = src[e];
     if (c == 1) {
-      a.dst.p[gi][to] = val;
-      a.dst_m.p[gi][to] = a.src_m.p[gi][from];
-      a.dst_v.p[gi][to] = a.src_v.p[gi][from];
+      const V vm = src_m[e], vv = src_v[e];
+      dst[to] = val;
+      dst_m[to] = vm;
+      dst_v[to] = vv;
       continue;
     }
-    float v0 = val, v1 = val;
-    if (gi <= 1) {  // split along the longest axis
-      const float* ls = a.src.p[1] + 3 * i;
-      const int ax = ls[0] >= ls[1] ? (ls[0] >= ls[2] ? 0 : 2) : (ls[1] >= ls[2] ? 1 : 2);
+    V v0 = val, v1 = val;
+    if constexpr (W == 3) {  // (means and log-scales; degree-0 colours are copied)
       if (gi == 0) {
-        float r3[3];
-        quat_axis(a.src.p[2] + 4 * i, ax, r3);
-        const float half = 0.5f * expf(ls[ax]);
-        const float d = half * (k == 0 ? r3[0] : (k == 1 ? r3[1] : r3[2]));
-        v0 = val + d;
-        v1 = val - d;
-      } else if (k == ax) {
+        v0 = fmaf(rows.half[r], rows.along[r][k], val);
+        v1 = fmaf(-rows.half[r], rows.along[r][k], val);
+      } else if (gi == 1 && k == rows.axis[r]) {
         v0 = v1 = val + logf(0.8660254037844386f);  // sigma_a sqrt(3)/2
       }
     }
-    a.dst.p[gi][to] = v0;
-    a.dst.p[gi][to + W] = v1;
-    a.dst_m.p[gi][to] = a.dst_m.p[gi][to + W] = 0.f;
-    a.dst_v.p[gi][to] = a.dst_v.p[gi][to + W] = 0.f;
+    dst[to] = v0;
+    dst[to + E] = v1;
+    dst_m[to] = dst_m[to + E] = V{};
+    dst_v[to] = dst_v[to + E] = V{};
   }
 }
 
-__global__ void __launch_bounds__(kApplyThreads) densify_apply_kernel(DensifyArgs a, const uint32_t* __restrict__ outc,
-                                                                      const uint32_t* __restrict__ pos, int64_t n) {
+// Bound by HBM: three arrays read and written, 59 floats a Gaussian at degree 3.
+__global__ void __launch_bounds__(kApplyThreads) densify_apply_kernel(DensifyArgs a, const uint32_t* __restrict__ plan,
+                                                                      const uint64_t* __restrict__ bases,
+                                                                      const DensifyTotals* __restrict__ totals, int64_t n) {
+  static_assert(kPlanBlock % kApplyRows == 0, "a CTA's rows lie in one block of the plan");
+  pdl_wait();
+  __shared__ ApplyRows rows;
   const int64_t i0 = (int64_t)blockIdx.x * kApplyRows;
-  apply_array<3>(a, 0, outc, pos, i0, n);
-  apply_array<3>(a, 1, outc, pos, i0, n);
-  apply_array<4>(a, 2, outc, pos, i0, n);
-  apply_array<1>(a, 3, outc, pos, i0, n);
+  const int n_rows = (int)(n - i0 < kApplyRows ? n - i0 : kApplyRows);
+  if ((int)threadIdx.x < n_rows) {
+    const int r = threadIdx.x;
+    const int64_t i = i0 + r;
+    const uint32_t word = plan[i], d = word >> (2 * kPlanBits);
+    const uint64_t base = bases[i0 / kPlanBlock];
+    const uint32_t allowed = (uint32_t)totals->allowed;
+    const uint32_t candidates = (uint32_t)(base >> 32) + (word >> kPlanBits & kPlanMask);
+    const uint32_t copies = d == 0 ? 0u : (d == 2 && candidates < allowed ? 2u : 1u);
+    rows.copies[r] = copies;
+    rows.to[r] = (uint32_t)base + (word & kPlanMask) + min(candidates, allowed);
+    if (copies == 2) {  // along the longest axis
+      const float* ls = a.src.p[1] + 3 * i;
+      const int ax = ls[0] >= ls[1] ? (ls[0] >= ls[2] ? 0 : 2) : (ls[1] >= ls[2] ? 1 : 2);
+      float r3[3];
+      quat_axis(a.src.p[2] + 4 * i, ax, r3);
+      rows.axis[r] = ax;
+      rows.half[r] = 0.5f * expf(ls[ax]);
+      for (int k = 0; k < 3; ++k) rows.along[r][k] = r3[k];
+    }
+  }
+  __syncthreads();
+  apply_array<3, float>(a, 0, rows, i0, n_rows);
+  apply_array<3, float>(a, 1, rows, i0, n_rows);
+  if (a.vec[2]) apply_array<4, float4>(a, 2, rows, i0, n_rows);
+  else apply_array<4, float>(a, 2, rows, i0, n_rows);
+  apply_array<1, float>(a, 3, rows, i0, n_rows);
   switch (a.K3) {
-    case 3: apply_array<3>(a, 4, outc, pos, i0, n); break;
-    case 12: apply_array<12>(a, 4, outc, pos, i0, n); break;
-    case 27: apply_array<27>(a, 4, outc, pos, i0, n); break;
-    default: apply_array<48>(a, 4, outc, pos, i0, n);
+    case 3: apply_array<3, float>(a, 4, rows, i0, n_rows); break;
+    case 12:
+      if (a.vec[4]) apply_array<12, float4>(a, 4, rows, i0, n_rows);
+      else apply_array<12, float>(a, 4, rows, i0, n_rows);
+      break;
+    case 27: apply_array<27, float>(a, 4, rows, i0, n_rows); break;
+    default:
+      if (a.vec[4]) apply_array<48, float4>(a, 4, rows, i0, n_rows);
+      else apply_array<48, float>(a, 4, rows, i0, n_rows);
   }
 }
 
@@ -313,36 +412,19 @@ NGS_API int ngs_densify(ngs_ctx* ctx, int64_t n, int32_t sh_degree, const ngs_gr
     return fail(ctx, NGS_ERR_INVALID_ARG, "densify: null array");
   cudaStream_t s = (cudaStream_t)stream;
   const uint32_t un = (uint32_t)n;
-  // scratch: decision, candidate flags, their scan, output counts, their scan, identity order (u32 each),
-  // allowed count; the scan's block sums and totals in the context's scan scratch
-  const size_t words = 6 * ((size_t)un + 1) + 4;
-  int rc = ensure(ctx, ctx->densify_tmp, sizeof(uint32_t) * words);
-  if (rc == NGS_OK) rc = ensure(ctx, ctx->scan_tmp, sizeof(uint64_t) * scan_tmp_words(un));
-  if (rc == NGS_OK) rc = ensure(ctx, ctx->densify_totals, 3 * sizeof(uint64_t));
+  // scratch: the plan words; the totals and the blocks' first places
+  const unsigned plan_blocks = (un + kPlanBlock - 1) / kPlanBlock;
+  int rc = ensure(ctx, ctx->densify_tmp, sizeof(uint32_t) * (size_t)un);
+  const size_t had = ctx->densify_totals.cap;
+  if (rc == NGS_OK) rc = ensure(ctx, ctx->densify_totals, sizeof(DensifyTotals) + sizeof(uint64_t) * plan_blocks);
   if (rc != NGS_OK) return rc;
-  uint32_t* decision = ctx->densify_tmp.as<uint32_t>();
-  uint32_t* cand = decision + (un + 1);
-  uint32_t* rank = cand + (un + 1);
-  uint32_t* outc = rank + (un + 1);
-  uint32_t* pos = outc + (un + 1);
-  uint32_t* iota = pos + (un + 1);
-  uint32_t* allowed = iota + (un + 1);
-  uint64_t* totals = ctx->densify_totals.as<uint64_t>();
-  const unsigned blocks = (un + 255) / 256;
-  int launches = 0;
-  iota_kernel<<<blocks, 256, 0, s>>>(iota, n);
-  densify_decide_kernel<<<blocks, 256, 0, s>>>(params->d_opacity_logits, params->d_log_scales, accum, count, n, *cfg,
-                                               decision, cand);
-  launches += 2;
-  cudaError_t me = launch_scan_counts(cand, iota, un, rank, ctx->scan_tmp.as<uint64_t>(), &totals[0], s, &launches);
-  if (me == cudaSuccess) me = cudaMemsetAsync(&totals[1], 0, sizeof(uint64_t), s);
+  uint32_t* plan = ctx->densify_tmp.as<uint32_t>();
+  DensifyTotals* totals = ctx->densify_totals.as<DensifyTotals>();
+  uint64_t* bases = reinterpret_cast<uint64_t*>(totals + 1);
+  const cudaError_t me = ctx->densify_totals.cap == had ? cudaSuccess : cudaMemsetAsync(totals, 0, sizeof(DensifyTotals), s);
   if (me != cudaSuccess) return fail(ctx, NGS_ERR_CUDA, std::string("densify: ") + cudaGetErrorString(me));
-  count_pruned_kernel<<<blocks, 256, 0, s>>>(decision, n, &totals[1]);
-  densify_allowed_kernel<<<1, 1, 0, s>>>(&totals[0], &totals[1], n, cfg->max_gaussians, allowed);
-  densify_count_kernel<<<blocks, 256, 0, s>>>(decision, rank, allowed, n, outc);
-  launches += 3;
-  me = launch_scan_counts(outc, iota, un, pos, ctx->scan_tmp.as<uint64_t>(), &totals[2], s, &launches);
-  if (me != cudaSuccess) return fail(ctx, NGS_ERR_CUDA, std::string("densify: ") + cudaGetErrorString(me));
+  launch_pdl(densify_plan_kernel, plan_blocks, kPlanThreads, 0, s, params->d_opacity_logits, params->d_log_scales, accum,
+             count, n, *cfg, plan, bases, totals, ctx->d_h_total + kMirrorDensify);
   DensifyArgs da;
   da.src = ptrs(*params);
   da.src_m = ptrs(*m);
@@ -350,12 +432,13 @@ NGS_API int ngs_densify(ngs_ctx* ctx, int64_t n, int32_t sh_degree, const ngs_gr
   da.dst = ptrs(*out_params);
   da.dst_m = ptrs(*out_m);
   da.dst_v = ptrs(*out_v);
+  for (int k = 0; k < 5; ++k)
+    da.vec[k] = (((uintptr_t)da.src.p[k] | (uintptr_t)da.src_m.p[k] | (uintptr_t)da.src_v.p[k] | (uintptr_t)da.dst.p[k] |
+                  (uintptr_t)da.dst_m.p[k] | (uintptr_t)da.dst_v.p[k]) & 15) == 0;
   da.K3 = 3 * (sh_degree + 1) * (sh_degree + 1);
-  densify_apply_kernel<<<(unsigned)((n + kApplyRows - 1) / kApplyRows), kApplyThreads, 0, s>>>(da, outc, pos, n);
-  launches += 1;
-  ctx->launches += launches;
-  publish_words(ctx, &totals[2], 1, kMirrorDensify, s);  // the new count, through the mapped mirror
-  ctx->launches += 1;
+  launch_pdl(densify_apply_kernel, (unsigned)((n + kApplyRows - 1) / kApplyRows), kApplyThreads, 0, s, da, plan, bases,
+             totals, n);
+  ctx->launches += 2;
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return fail(ctx, NGS_ERR_CUDA, std::string("densify: ") + cudaGetErrorString(e));

@@ -91,6 +91,39 @@ def test_densify_matches_oracle(rnd):
                                    rtol=0, atol=0, err_msg=k)
 
 
+@pytest.mark.parametrize("n", [1, 63, 64, 1024, 1025, 3001])  # the blocks of the plan and of the moved rows
+@pytest.mark.parametrize("degree,shift", [(0, 0), (1, 0), (1, 1), (2, 0), (3, 0), (3, 1)])  # shift: rows off 16 bytes
+def test_densify_sizes_and_caps_match_oracle(rnd, n, degree, shift):
+    rng = np.random.default_rng(n + degree)
+    p = {"means": rng.standard_normal((n, 3)), "log_scales": rng.normal(-4, 1.5, (n, 3)),
+         "quats": rng.standard_normal((n, 4)), "opacity_logits": rng.normal(-1, 3, n),
+         "sh": rng.standard_normal((n, (degree + 1) ** 2, 3))}
+    p = {k: v.astype(np.float32) for k, v in p.items()}
+    m = {k: rng.standard_normal(v.shape).astype(np.float32) for k, v in p.items()}
+    vv = {k: rng.random(v.shape).astype(np.float32) for k, v in p.items()}
+    accum = (rng.random(n) * 2e-3).astype(np.float32)
+    count = rng.integers(0, 4, n).astype(np.float32)
+
+    def device(a):
+        t = torch.empty(a.size + 4, device="cuda")[shift:shift + a.size].view(a.shape)
+        return t.copy_(torch.from_numpy(a))
+
+    # no room, room for some candidates, room for all; splits or prunes alone
+    for cap, split, prune in ((0, True, True), (n, True, True), (n + n // 8, True, True), (2 * n, True, False),
+                              (2 * n, False, True)):
+        adam = Adam({k: device(v) for k, v in p.items()})
+        adam.m, adam.v = ({k: device(v) for k, v in d.items()} for d in (m, vv))
+        out = densify(rnd, {k: device(v) for k, v in p.items()}, adam, device(accum), device(count),
+                      grad_threshold=3e-4, max_gaussians=cap, split=split, prune=prune)
+        want = T.densify({k: v.astype(np.float64) for k, v in p.items()}, m, vv, accum.astype(np.float64),
+                         count.astype(np.float64), 3e-4, 0.008, 1e-4, cap, split=split, prune=prune)
+        assert out["means"].shape[0] == len(want[0]["means"])
+        for k in PARAM_KEYS:
+            for got, ref, tol in ((out[k], want[0][k], 1e-5), (adam.m[k], want[1][k], 0), (adam.v[k], want[2][k], 0)):
+                np.testing.assert_allclose(got.cpu().numpy().reshape(-1), ref.reshape(-1), rtol=tol, atol=tol / 10,
+                                           err_msg=k)
+
+
 @pytest.fixture(scope="module")
 def recon(rnd):
     gt = upload(synth.clustered_scene(6000, seed=21, sh_degree=1, box=4.0))
