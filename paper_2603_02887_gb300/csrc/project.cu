@@ -408,12 +408,21 @@ __device__ __forceinline__ uint2 count_listed(RowList& list, const SplatBin& b, 
 // A splat spanning more tile rows than this has them counted by its whole warp, one row per lane.
 constexpr int kCoopRows = 8;  // (the rows of a tile mask)
 
-// Block b works on view b % n_views and Gaussians [256 (b / n_views), +256): the views of one block of
+// Block b works on view b % n_views and Gaussians [128 (b / n_views), +128): the views of one block of
 // Gaussians run side by side, so their parameters are read from HBM once and from L2 afterwards.
 // A single view takes its camera from the kernel parameters (cam0), a batch (or a captured graph, which
 // must serve any pose) from the view table; the arithmetic below is the same code either way.
+//
+// 16-byte SH rows (VEC): a warp brings its 32 Gaussians' rows, contiguous in memory, into shared memory with coalesced
+// loads, and each lane reads its own there (rows an odd number of 16-byte words apart: no bank conflicts). A lane reading its own row of
+// 192 bytes from global memory touched 32 lines an instruction, 384 cycles of the L1 pipe a warp, which was the
+// kernel's busiest unit (76 %). The same shared memory lists the tile rows afterwards. Seven CTAs of 128 per SM at 72
+// registers: 500k, 1920x1080 on 16 x 16 tiles 59 -> 53 us (with the frame's start), 1M, 1297x840 112 -> 100 us, 8 views of 1M
+// 558 -> 433 us, 32 views of 3M on 8 x 8 tiles 7.92 -> 6.26 ms (eight CTAs, 64 registers and 54 bytes of spills: 7.07 ms,
+// six: 7.12 ms).
+constexpr int kProjThreads = 128;
 template <int DEG, bool VEC, bool BINS>
-__global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const ViewParams* __restrict__ views,
+__global__ void __launch_bounds__(kProjThreads, 7) project_kernel(ngs_gaussians g, const ViewParams* __restrict__ views,
                                                       CamParams cam0, RenderParams rp, float4* rec,
                                                       uint32_t* depth_key, uint32_t* tile_count, uint32_t* order,
                                                       uint2* bins, TileMasks masks) {
@@ -427,18 +436,35 @@ __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const 
     if constexpr (BINS) bins += views[view].tile_base;
   }
   const int64_t r = (int64_t)view * g.n + i;  // record index
+  RawParams prm;
   if (i < g.n) {
-    // every line the projection reads, requested at once: the loads behind the depth test and inside the
-    // colour find them in L1 instead of making three round trips to memory one after another
-    prefetch_l1(g.means + 3 * (int64_t)i);
-    prefetch_l1(g.log_scales + 3 * (int64_t)i);
-    prefetch_l1(g.quats + 4 * (int64_t)i);
-    prefetch_l1(g.opacity_logits + i);
-    const char* sh = reinterpret_cast<const char*>(g.sh + (int64_t)i * ProjState<DEG>::K * 3);
-    constexpr int kShBytes = ProjState<DEG>::K * 3 * 4;
+    if constexpr (!VEC) {  // its SH lines, requested before the depth test
+      const char* sh = reinterpret_cast<const char*>(g.sh + (int64_t)i * ProjState<DEG>::K * 3);
+      constexpr int kShBytes = ProjState<DEG>::K * 3 * 4;
 #pragma unroll
-    for (int o = 0; o < kShBytes; o += 128) prefetch_l1(sh + o);
-    prefetch_l1(sh + kShBytes - 4);
+      for (int o = 0; o < kShBytes; o += 128) prefetch_l1(sh + o);
+      prefetch_l1(sh + kShBytes - 4);
+    }
+    prm = load_params(g, i);
+  }
+  constexpr int Q = VEC ? 3 * ProjState<DEG>::K / 4 : 1, kRow = Q | 1;  // float4 of a row, and between rows
+  constexpr int kShWords = VEC ? 32 * kRow : 1, kListWords = BINS ? (int)(sizeof(RowList) / sizeof(float4)) : 1;
+  __shared__ float4 s_warp[kProjThreads / 32][kShWords > kListWords ? kShWords : kListWords];
+  float4* const warp_mem = s_warp[threadIdx.x >> 5];
+  if constexpr (VEC) {
+    const int g0 = i - lane;  // the warp's first Gaussian
+    const float4* const src = reinterpret_cast<const float4*>(g.sh) + (int64_t)g0 * Q;
+    const int words = min((int)g.n - g0, 32) * Q;
+    float4 w[Q];
+#pragma unroll
+    for (int k = 0; k < Q; ++k)
+      if (k * 32 + lane < words) w[k] = src[k * 32 + lane];
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      const int idx = k * 32 + lane, row = idx / Q;
+      if (idx < words) warp_mem[row * kRow + (idx - row * Q)] = w[k];
+    }
+    __syncwarp();
   }
   // every lane stays to the end: the warp counts its tall splats' tiles together
   uint32_t count = 0;
@@ -449,12 +475,13 @@ __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const 
   float z = 0.f;
   if (i < g.n) {
     const CamParams cam = rp.cam_from_table ? views[view].cam : cam0;
-    const float* m = g.means + 3 * (int64_t)i;
-    z = view_depth(cam, m[0], m[1], m[2]);
+    z = view_depth(cam, prm.m[0], prm.m[1], prm.m[2]);
     float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f), r1 = r0, r2 = make_float4(0.f, z, 0.f, 0.f);
     if (z > rp.near_plane) {
       ProjState<DEG> st;
-      forward_map<DEG, VEC>(load_params(g, i), cam, rp, st, g.sh + (int64_t)i * ProjState<DEG>::K * 3);
+      forward_map<DEG, VEC>(prm, cam, rp, st,
+                            VEC ? reinterpret_cast<const float*>(warp_mem + lane * kRow)
+                                : g.sh + (int64_t)i * ProjState<DEG>::K * 3);
       if (st.det > 0.f && st.aleph >= rp.alpha_min && isfinite(st.A) && isfinite(st.C)) {
         float u = cam.fx * st.x * st.iz + cam.cx;
         float v = cam.fy * st.y * st.iz + cam.cy;
@@ -484,8 +511,9 @@ __global__ void __launch_bounds__(256, 4) project_kernel(ngs_gaussians g, const 
     if constexpr (!BINS) order[r] = (uint32_t)r;
   }
   if constexpr (BINS) {
-    __shared__ __align__(16) RowList s_rows[8];
-    mask = count_listed(s_rows[threadIdx.x >> 5], b, rp, boxed, x0, x1, y0, y1, bins);
+    static_assert(sizeof(RowList) % sizeof(float4) == 0, "whole words");
+    __syncwarp();  // the SH rows have been read
+    mask = count_listed(*reinterpret_cast<RowList*>(warp_mem), b, rp, boxed, x0, x1, y0, y1, bins);
     count = (uint32_t)(__popc(mask.x) + __popc(mask.y));
   }
   // tall splats, one after another: lane l counts tile rows y0 + l, y0 + l + 32, ... (the same row spans)
@@ -1064,10 +1092,10 @@ void launch_project(const ngs_gaussians& g, const ViewParams* views, const CamPa
                     float4* rec, uint32_t* depth_key, uint32_t* tile_count, uint32_t* order, uint2* bins,
                     const TileMasks& masks, cudaStream_t s) {
   if (g.n == 0) return;
-  unsigned blocks = (unsigned)((g.n + 255) / 256) * rp.n_views;
+  unsigned blocks = (unsigned)((g.n + kProjThreads - 1) / kProjThreads) * rp.n_views;
   bool vec = ((uintptr_t)g.sh & 15) == 0;
 #define NGS_PROJECT(D, V)                                                                                            \
-  launch_pdl(bins ? project_kernel<D, V, true> : project_kernel<D, V, false>, blocks, 256, 0, s, g, views, cam0, rp, rec, \
+  launch_pdl(bins ? project_kernel<D, V, true> : project_kernel<D, V, false>, blocks, kProjThreads, 0, s, g, views, cam0, rp, rec, \
              depth_key, tile_count, order, bins, masks)
   switch (rp.sh_degree) {
     case 0: NGS_PROJECT(0, false); break;

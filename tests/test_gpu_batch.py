@@ -327,3 +327,25 @@ def test_batch_parameter_gradients_are_the_views_sums(rnd, n, degree):
             rnd.recycle(f)
         for k, g in grads.items():  # FP32 sums of four views and of their pixels in another order
             assert torch.allclose(g.double(), total[k].view_as(g), rtol=1e-4, atol=1e-5 * scale[k] + 1e-12), k
+
+
+@pytest.mark.parametrize("degree", [1, 3])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 127, 129, 300])
+def test_rows_staged_and_not_project_alike(rnd, n, degree):
+    """SH rows on 16-byte boundaries go through shared memory a warp at a time, others are read by their own thread: the
+    same records, for warps and blocks that are not full, in one view and in three."""
+    scene = synth.clustered_scene(n, seed=n, sh_degree=degree)
+    cams = [synth.outside_camera(64, 48, 12.0), synth.outside_camera(40, 40, 0.5), synth.outside_camera(33, 70, 9.0)]
+    got = []
+    for shift in (0, 1):
+        params = upload(scene)
+        store = torch.empty(params["sh"].numel() + 4, device="cuda")
+        sh = store[shift:shift + params["sh"].numel()].view_as(params["sh"])
+        params["sh"] = sh.copy_(params["sh"])
+        for views in (cams[:1], cams):
+            _, _, frame = rnd.render_batch(params, views, "sup")
+            got.append(batch_arrays(frame)["records"])
+            rnd.recycle(frame)
+    for a, b in zip(got[:2], got[2:]):  # the colour's 16 terms may be contracted another way
+        assert np.allclose(a, b, rtol=1e-5, atol=1e-6)
+    assert np.array_equal(_bits(got[0]), _bits(got[1][:n]))
