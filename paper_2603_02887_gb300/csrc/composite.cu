@@ -6,8 +6,8 @@
 // Replay, and the forward of the exponential model (and of the quadratic ones on tiles of >= 256 pixels):
 // two pixels per thread, (x, y) and (x, y + 4), so that a warp covers an 8 x 8 block; the two step through
 // each entry together in packed FP32x2 instructions (add / mul / fma .rn.f32x2), each lane rounding like
-// the one-pixel form, with splat operands staged in duplicated pairs. The replay sums its contributions over
-// the 64 pixels for eight entries at a time. Other forwards: one thread per pixel, warps on 8 x 4 pixel blocks
+// the one-pixel form, with the splat operands staged in duplicated pairs. The replay reduces both pixels'
+// contributions once per 64 pixels. Other forwards: one thread per pixel, warps on 8 x 4 pixel blocks
 // whose pixels are close and tend to saturate together.
 //
 // Forward, per pixel (Eq. generalized_gaussian with pbar_i from Eq. nexp_p and Table 1):
@@ -30,9 +30,9 @@
 //                of DeltaE_l alpha_l P_l and B their total (saved by the forward pass);
 //   Vicini:      (1 - g) x the linear adjoint + g x the exponential adjoint, each over its own list;
 // then w = dL/d(log2 alpha) and its moments w, w dx, w dy, w dx^2, w dx dy, w dy^2 (which determine the
-// gradient of the splat record, see the projection backward) and dL/dE: a warp gathers the w and pbar of eight
-// entries in shared memory, sums them over its pixels four lanes to an entry, and adds the totals to the
-// per-Gaussian buffer.
+// gradient of the splat record, see the projection backward) and dL/dE: added to the per-Gaussian buffer by
+// each lane that hit the splat when at most kDirectLanes did, else reduced over the warp with shuffles and
+// added with one atomic-add instruction per value.
 #include <algorithm>
 
 #include <type_traits>
@@ -79,6 +79,11 @@ struct TileGeom {
 // The forward keeps one pixel per thread (a thread retires with its pixel); the replay takes two, so that
 // the warp reduces once per 64 pixels.
 constexpr int kBwdPix = 2;
+// Replay: a splat hit by at most this many lanes of a warp is added by those lanes directly; more go through
+// the warp reduction (32 atomics on one address serialise). Measured on GB300 with the packed replay at
+// 500k Gaussians / 1080p: on 8x8 tiles 16 beats 8, 12, 24 and 32 (exponential replay 0.351 ms against
+// 0.379 at 24 and 0.80 at 32), on 16x16 tiles 16 and 24 tie.
+constexpr int kDirectLanes = 16;
 
 // ---- forward ---------------------------------------------------------------------------------------
 
@@ -118,28 +123,26 @@ __device__ __forceinline__ uint32_t next_tile(const uint32_t* __restrict__ work,
   return w < n_tiles ? (work ? work[w] : w) : n_tiles;
 }
 
-// Staging of one chunk for the packed (two pixels per thread) forward and replay. The operands of FP32x2 instructions
-// are duplicated: one 16-byte shared load gives the operand pairs {a, a, b, b} of two instructions. The replay
-// keeps only C' and L so, and takes its other operands single, in scalar instructions (see kSlots).
-template <int CH, bool REPLAY>
-struct PairStageBuf {  // (the first arrays have an entry that is read ahead but never used)
-  float4 r0[REPLAY ? CH + 1 : 1];  // replay: {u, v, A', B'}
-  float4 q0[REPLAY ? 1 : CH + 1];  // forward: {-u, -u, -v, -v}
-  float4 q1[REPLAY ? 1 : CH + 1];  // forward: {A', A', B', B'}
+// Staging of one chunk for the packed (two pixels per thread) forward and replay: every per-splat operand
+// duplicated, so one 16-byte shared load gives the operand pairs {a, a, b, b} of two FP32x2 instructions.
+template <int CH>
+struct PairStageBuf {  // (q0..q2 have an entry that is read ahead but never used)
+  float4 q0[CH + 1];  // {-u, -u, -v, -v}
+  float4 q1[CH + 1];  // {A', A', B', B'}
   float4 q2[CH + 1];  // {C', C', L, L}
-  float4 q3[CH];  // forward: {E0, E0, E1, E1}; replay: {E0, E1, E2, record index (bits)}
-  float2 q4[REPLAY ? 1 : CH];  // forward: {E2, E2}
+  float4 q3[CH];  // {E0, E0, E1, E1}
+  float4 q4[CH];  // {E2, E2, record index (bits), 0}: one 16-byte load gives E2 and the atomics' target
 };
 
-// The packed form (exponential and quadratic models) is used while the forward's staging (72 B per record) stays
+// The packed form (exponential and quadratic models) is used while its staging (72 B per record) stays
 // within 40 KB of static shared memory.
 template <int KIND, int CH>
-constexpr bool kPairForm = (KIND == NGS_MODEL_EXP || KIND == NGS_MODEL_QUAD) && sizeof(PairStageBuf<CH, false>) <= 41248;
+constexpr bool kPairForm = (KIND == NGS_MODEL_EXP || KIND == NGS_MODEL_QUAD) && sizeof(PairStageBuf<CH>) <= 41216;
 
-template <int B, int CH, bool REPLAY>
+template <int B, int CH>
 __device__ __forceinline__ void stage_chunk_pairs(const float4* __restrict__ rec, const uint32_t* __restrict__ ids,
                                                   const RenderParams& rp, uint32_t base, uint32_t end,
-                                                  PairStageBuf<CH, REPLAY>& sb) {
+                                                  PairStageBuf<CH>& sb) {
 #pragma unroll
   for (int k = 0; k < (CH + B - 1) / B; ++k) {
     const int slot = k * B + (int)threadIdx.x;
@@ -149,19 +152,11 @@ __device__ __forceinline__ void stage_chunk_pairs(const float4* __restrict__ rec
       float4 r0, r1;
       float e2;
       stage_record(rec, id, rp, r0, r1, e2);
-      if constexpr (REPLAY) {
-        sb.r0[slot] = r0;
-      } else {
-        sb.q0[slot] = make_float4(-r0.x, -r0.x, -r0.y, -r0.y);
-        sb.q1[slot] = make_float4(r0.z, r0.z, r0.w, r0.w);
-      }
+      sb.q0[slot] = make_float4(-r0.x, -r0.x, -r0.y, -r0.y);
+      sb.q1[slot] = make_float4(r0.z, r0.z, r0.w, r0.w);
       sb.q2[slot] = make_float4(r1.x, r1.x, r1.y, r1.y);
-      if constexpr (REPLAY) {
-        sb.q3[slot] = make_float4(r1.z, r1.w, e2, __uint_as_float(id < rp.n_records ? id : 0u));
-      } else {
-        sb.q3[slot] = make_float4(r1.z, r1.z, r1.w, r1.w);
-        sb.q4[slot] = make_float2(e2, e2);
-      }
+      sb.q3[slot] = make_float4(r1.z, r1.z, r1.w, r1.w);
+      sb.q4[slot] = make_float4(e2, e2, __uint_as_float(id < rp.n_records ? id : 0u), 0.f);
     }
   }
 }
@@ -354,7 +349,7 @@ __device__ __forceinline__ void forward_tile_pairs(const float4* __restrict__ re
                                                    const uint2* __restrict__ ranges, const RenderParams& rp,
                                                    const ViewParams* __restrict__ views, float* __restrict__ image,
                                                    int32_t* __restrict__ overdraw, float4* __restrict__ state,
-                                                   uint32_t tile, PairStageBuf<CH, false>& sb) {
+                                                   uint32_t tile, PairStageBuf<CH>& sb) {
   using G = TileGeom<TW, TH, 2>;
   constexpr int B = G::kThreads;
   const TileView tv = tile_view(rp, views, (uint32_t)tile);
@@ -411,7 +406,7 @@ __device__ __forceinline__ void forward_tile_pairs(const float4* __restrict__ re
           continue;
         }
         const float4 q3 = sb.q3[j];
-        const float2 E0 = lo_hi(q3, false), E1 = lo_hi(q3, true), E2 = sb.q4[j];
+        const float2 E0 = lo_hi(q3, false), E1 = lo_hi(q3, true), E2 = lo_hi(sb.q4[j], false);
         const float2 alpha = make_float2(on0 ? fminf(amax, fast_exp2(e.x)) : 0.f, on1 ? fminf(amax, fast_exp2(e.y)) : 0.f);
         const uint32_t pos = base + j - range.x;
         bool c0, c1;  // composited (the overdraw count)
@@ -546,7 +541,7 @@ __global__ void __launch_bounds__(kFwdThreads<TW, TH, KIND, CH>, kFwdMinBlocks<T
                                                                    const uint32_t* __restrict__ work,
                                                                    uint32_t* counter) {
   pdl_wait();
-  using Buf = std::conditional_t<kPairFwd<TW, TH, KIND, CH>, PairStageBuf<CH, false>, StageBuf<CH>>;
+  using Buf = std::conditional_t<kPairFwd<TW, TH, KIND, CH>, PairStageBuf<CH>, StageBuf<CH>>;
   __shared__ Buf sb;
   auto one_tile = [&](uint32_t tile) {
     if constexpr (kPairFwd<TW, TH, KIND, CH>)
@@ -578,99 +573,51 @@ struct BwdPixel {
   bool sat, stop_e;     // Vicini: the linear list saturated / the exponential list stopped
 };
 
-// ---- replay: sums over a warp's pixels ----------------------------------------------------------------
-//
-// A warp holds each composited entry's w = dL/d(log2 alpha) (over ln 2) and wE = dL0/dE of its 64 pixels, 16 B per
-// lane, until kSlots entries have gathered; then lane (r, e) sums entry e over the pixel rows r and r + 4, and the four
-// lanes of an entry add their sums. About 16 instructions an entry, and 9 atomics in two instructions. Reducing each
-// entry by itself took about 50: nine sums through twelve shuffles, or up to 16 lanes' own atomics, whichever were fewer.
-// Eight entries are the most whose words leave the registers, not shared memory, to limit a multiprocessor's warps (28).
-// What bounds the walk now are the shared-memory pipe (82 % busy) and the issue slots (70 %): a 16-byte load takes two of the pipe's cycles
-// even where all lanes read the same words, which is why the replay stages its operands single (273 us; duplicated for
-// the packed instructions as in the forward: 326 us). Replay before -> now: 500k, 1920x1080, exponential on 8 x 8 tiles
-// 326 -> 273 us, c = -0.5 on 16 x 16 147 -> 133 us; 1M, 1297x840, c = 0 101 -> 96 us; 32 views of 3M 9.29 -> 8.2 ms;
-// 1k, 128x128 27 -> 22 us.
-constexpr int kSlots = 8;
-constexpr int kSlotStride = 33;  // float4: eight lanes read eight entries without bank conflicts
-
-struct ReplayWarp {
-  float4 w[kSlots * kSlotStride];  // [entry][lane]: {w, w, wE, wE} of pixels (x, y) and (x, y + 4)
-  float4 g01[32];                  // [lane]: {g0, g0, g1, g1} of the two pixels
-  float2 g2[32];
-};
-
-// The entry in slot lane % kSlots, held by each of its four lanes.
-struct ReplaySlot {
-  float u, v;
-  uint32_t id;  // record index
-};
-
-// The replay of a warp's 8 x 8 block starts: the upstream gradients of the thread's two pixels. A lane with one that
-// is not finite (returned) adds its own products to dL/dE (replay_odd_lane), so that it reaches only the entries it composites.
-__device__ __forceinline__ bool replay_begin(ReplayWarp& rw, const float (&ga)[3], const float (&gb)[3], int lane) {
-  const bool odd = !(isfinite(ga[0]) && isfinite(ga[1]) && isfinite(ga[2]) && isfinite(gb[0]) && isfinite(gb[1]) &&
-                     isfinite(gb[2]));
-  rw.g01[lane] = odd ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(ga[0], gb[0], ga[1], gb[1]);
-  rw.g2[lane] = odd ? make_float2(0.f, 0.f) : make_float2(ga[2], gb[2]);
-  return odd;
-}
-
-__device__ __forceinline__ void replay_odd_lane(float* dst, float g0, float g1, float g2, float wE) {
-  atomicAdd(dst + 6, g0 * wE);
-  atomicAdd(dst + 7, g1 * wE);
-  atomicAdd(dst + 8, g2 * wE);
-}
-
-// Adds the sums of the first `count` gathered entries to grad2d: the moments w dx, w dy, w dx^2, w dx dy, w dy^2, w
-// and the three of dL/dE. (bx, by): the centre of the block's first pixel.
-__device__ __forceinline__ void replay_flush(const ReplayWarp& rw, const ReplaySlot& slot, uint32_t count, float bx,
-                                             float by, float4* __restrict__ grad2d, int lane) {
-  __syncwarp();
-  const uint32_t e = lane & 7, r = lane >> 3;
-  const float2 one = make_float2(1.f, 1.f), zero = make_float2(0.f, 0.f);
-  const float2 dy = __fadd2_rn(make_float2(by + (float)r, by + (float)(r + 4)), make_float2(-slot.v, -slot.v));
-  float2 dx = __fadd2_rn(make_float2(bx, bx), make_float2(-slot.u, -slot.u));
-  float2 s0 = zero, s1 = zero, s2 = zero, c0 = zero, c1 = zero, c2 = zero;
-  const float4* w = rw.w + e * kSlotStride + 8 * r;
+// Sum nine per-lane values over the warp and add the totals to dst[0..8] with one atomic instruction.
+// Values 0..7 go through a transposing butterfly: at each of three steps a lane keeps half of the values
+// it carries and sends the other half to its partner, so after xor 16, 8, 4 a lane carries one of them,
+// summed over 8 lanes; value 8 is summed over the same lanes by a plain tree. The last two steps (xor 2,
+// 1) carry both, half of the lanes each, so that lane l ends with the warp total of value ((l >> 2) & 7)
+// when l % 4 == 0, and lane 2 with that of value 8: 12 shuffles instead of 45 for nine plain trees.
+__device__ __forceinline__ void warp_reduce9_add(const float (&v)[9], float* dst, int lane) {
+  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+  float w[4];
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const float4 ww = w[c], g01 = rw.g01[8 * r + c];
-    const float2 g2 = rw.g2[8 * r + c];
-    const float2 wgt = lo_hi(ww, false), wE = lo_hi(ww, true);
-    const float2 t = __fmul2_rn(wgt, dx);
-    s0 = __fadd2_rn(s0, wgt);
-    s1 = __fadd2_rn(s1, t);
-    s2 = __ffma2_rn(t, dx, s2);
-    c0 = __ffma2_rn(lo_hi(g01, false), wE, c0);
-    c1 = __ffma2_rn(lo_hi(g01, true), wE, c1);
-    c2 = __ffma2_rn(g2, wE, c2);
-    if (c < 7) dx = __fadd2_rn(dx, one);
+  for (int p = 0; p < 4; ++p) {
+    float send = b4 ? v[p] : v[p + 4];
+    float keep = b4 ? v[p + 4] : v[p];
+    w[p] = keep + __shfl_xor_sync(kFull, send, 16);
   }
-  const float2 wdy = __fmul2_rn(s0, dy), wdxdy = __fmul2_rn(s1, dy), wdydy = __fmul2_rn(wdy, dy);
-  const float v[9] = {s1.x + s1.y,       wdy.x + wdy.y, s2.x + s2.y, wdxdy.x + wdxdy.y, wdydy.x + wdydy.y,
-                      s0.x + s0.y,       c0.x + c0.y,   c1.x + c1.y, c2.x + c2.y};
-  // over the entry's four lanes, transposing: lane r ends with the totals 2 r and 2 r + 1
-  const bool b1 = r & 2, b0 = r & 1;
-  float x[4], y[2];
+  float x[2];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) x[k] = (b1 ? v[k + 4] : v[k]) + __shfl_xor_sync(kFull, b1 ? v[k] : v[k + 4], 16);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) y[k] = (b0 ? x[k + 2] : x[k]) + __shfl_xor_sync(kFull, b0 ? x[k] : x[k + 2], 8);
-  float z = v[8] + __shfl_xor_sync(kFull, v[8], 16);
-  z += __shfl_xor_sync(kFull, z, 8);
-  if (e < count) {
-    float* dst = reinterpret_cast<float*>(grad2d + 3 * (size_t)slot.id);
-    atomicAdd(reinterpret_cast<float2*>(dst + 2 * r), make_float2(y[0], y[1]));
-    if (r == 0) atomicAdd(dst + 8, z);
+  for (int p = 0; p < 2; ++p) {
+    float send = b3 ? w[p] : w[p + 2];
+    float keep = b3 ? w[p + 2] : w[p];
+    x[p] = keep + __shfl_xor_sync(kFull, send, 8);
   }
-  __syncwarp();  // the slots are free
+  float send = b2 ? x[0] : x[1];
+  float y = (b2 ? x[1] : x[0]) + __shfl_xor_sync(kFull, send, 4);
+  // the ninth value over lane bits 4..2, then both over bits 1 and 0 in one transposing step: lanes with
+  // bit 1 clear carry y, lanes with it set carry e
+  float e = v[8];
+  e += __shfl_xor_sync(kFull, e, 16);
+  e += __shfl_xor_sync(kFull, e, 8);
+  e += __shfl_xor_sync(kFull, e, 4);
+  const bool b1 = lane & 2;
+  float z = (b1 ? e : y) + __shfl_xor_sync(kFull, b1 ? y : e, 2);
+  z += __shfl_xor_sync(kFull, z, 1);
+  if ((lane & 3) == 0)
+    atomicAdd(dst + ((lane >> 2) & 7), z);  // value (lane >> 2) & 7, summed over the warp
+  else if ((lane & 3) == 2 && lane < 4)
+    atomicAdd(dst + 8, z);                  // the ninth, summed over the warp
 }
 
-// One list entry for one pixel of the replay: its w and wE (untouched where it does not composite the splat), and
-// whether it does.
+// One list entry for one pixel of the replay: adds the pixel's contributions to the per-splat sums that
+// do not involve dx (v[1], v[4..8]; the caller forms the dx moments once for the column) and returns
+// whether the splat was composited at this pixel.
 template <int KIND>
 __device__ __forceinline__ bool bwd_step(BwdPixel& p, float dx, float adx, float4 r0, float4 r1, const float& e2,
-                                         uint32_t pos, const RenderParams& rp, float& w_out, float& wE_out) {
+                                         uint32_t pos, const RenderParams& rp, float (&v)[9]) {
   if (pos >= p.last) return false;
   float dy;
   float e = splat_log2_alpha_col(dx, adx, p.py, r0, r1, dy);
@@ -751,8 +698,14 @@ __device__ __forceinline__ bool bwd_step(BwdPixel& p, float dx, float adx, float
   // w = dL/de, de/dA' = dx^2, de/dB' = dx dy, de/dC' = dy^2, de/dL = 1 and de/du = -(2A' dx + B' dy),
   // de/dv = -(B' dx + 2C' dy): the per-splat sums of w, w dx, w dy, w dx^2, w dx dy, w dy^2 carry
   // everything; the projection backward applies the per-splat A', B', C' (and ln 2) once.
-  w_out = raw >= rp.alpha_max ? 0.f : dLda * alpha;  // dL/de / ln 2
-  wE_out = wE;
+  float wgt = raw >= rp.alpha_max ? 0.f : dLda * alpha;  // dL/de / ln 2
+  float wdy = wgt * dy;
+  v[1] += wdy;
+  v[4] = fmaf(wdy, dy, v[4]);
+  v[5] += wgt;
+  v[6] = fmaf(p.g0, wE, v[6]);
+  v[7] = fmaf(p.g1, wE, v[7]);
+  v[8] = fmaf(p.g2, wE, v[8]);
   return true;
 }
 
@@ -766,8 +719,7 @@ __device__ __forceinline__ bool bwd_step(BwdPixel& p, float dx, float adx, float
 
 // Both pixels' replay state, lane 0 = pixel (x, y), lane 1 = pixel (x, y + 4).
 struct BwdPair {
-  float px;
-  float2 py;
+  float2 px, py;
   uint32_t last0, last1;  // replay entries [range.x, last)
   float2 g0, g1, g2;
   float2 T, gacc, gL0;    // exponential: T_i, g.sum_{j<i} E_j pbar_j, g.L0
@@ -775,30 +727,31 @@ struct BwdPair {
 };
 
 // The quadratic form of an entry at both pixels (as splat_log2_alpha_col computes it per pixel): e = log2
-// of aleph K.
-__device__ __forceinline__ float2 pair_log2_alpha(const BwdPair& p, float4 r0, float4 q2) {
-  const float dx = __fsub_rn(p.px, r0.x), adx = __fmul_rn(r0.z, dx);
-  const float2 dy = make_float2(__fsub_rn(p.py.x, r0.y), __fsub_rn(p.py.y, r0.y));
+// of aleph K, dx (px - u, equal in both lanes: one column) and dy.
+__device__ __forceinline__ float2 pair_log2_alpha(const BwdPair& p, float4 q0, float4 q1, float4 q2, float2& dx,
+                                                  float2& dy) {
+  dx = __fadd2_rn(p.px, lo_hi(q0, false));
+  const float2 adx = __fmul2_rn(lo_hi(q1, false), dx);
+  dy = __fadd2_rn(p.py, lo_hi(q0, true));
+  const float2 t = __ffma2_rn(lo_hi(q1, true), dy, adx);
   const float2 cdd = __fmul2_rn(__fmul2_rn(lo_hi(q2, false), dy), dy);
-  const float2 q = make_float2(__fmaf_rn(dx, __fmaf_rn(r0.w, dy.x, adx), cdd.x),
-                               __fmaf_rn(dx, __fmaf_rn(r0.w, dy.y, adx), cdd.y));
-  return __fadd2_rn(lo_hi(q2, true), q);
+  return __fadd2_rn(lo_hi(q2, true), __ffma2_rn(dx, t, cdd));
 }
 
 // One list entry for both pixels, given the quadratic form (e, dx, dy) and which pixels composite it
-// (on0 / on1: not past their stop, alpha >= alpha_min): {w, w, wE, wE}. A pixel that does not composite it gets
-// alpha = 0, which leaves its running sums exactly as they were, and zeros, so the warp runs the step
-// whenever any lane is on.
+// (on0 / on1: not past their stop, alpha >= alpha_min): adds their contributions to v (the 9 per-splat
+// sums, the dx moments included). A pixel that does not composite it gets alpha = 0, which leaves its
+// running sums exactly as they were and adds nothing, so the warp runs the step whenever any lane is on.
 template <int KIND>
-__device__ __forceinline__ float4 bwd_pair_step(BwdPair& p, float2 e, float4 q3, bool on0, bool on1,
-                                                const RenderParams& rp) {
+__device__ __forceinline__ void bwd_pair_step(BwdPair& p, float2 e, float2 dx, float2 dy, float4 q3, float4 q4,
+                                              bool on0, bool on1, const RenderParams& rp, float (&v)[9]) {
   const float2 one = make_float2(1.f, 1.f), neg = make_float2(-1.f, -1.f);
   const float raw0 = fast_exp2(e.x), raw1 = fast_exp2(e.y);
   const float2 alpha = make_float2(on0 ? fminf(rp.alpha_max, raw0) : 0.f, on1 ? fminf(rp.alpha_max, raw1) : 0.f);
   // w = dL/de: zero where alpha is clamped at alpha_max (it no longer depends on e) or not composited
   bool live0 = on0 && raw0 < rp.alpha_max, live1 = on1 && raw1 < rp.alpha_max;
-  const float2 gE = make_float2(fmaf(p.g2.x, q3.z, fmaf(p.g1.x, q3.y, p.g0.x * q3.x)),
-                                fmaf(p.g2.y, q3.z, fmaf(p.g1.y, q3.y, p.g0.y * q3.x)));
+  const float2 gE =
+      __ffma2_rn(p.g2, lo_hi(q4, false), __ffma2_rn(p.g1, lo_hi(q3, true), __fmul2_rn(p.g0, lo_hi(q3, false))));
   float2 dLda, wE;
   if constexpr (KIND == NGS_MODEL_QUAD) {
     const float2 ct = __ffma2_rn(make_float2(rp.c, rp.c), p.tau, one);  // 1 + c taubar_i
@@ -826,7 +779,18 @@ __device__ __forceinline__ float4 bwd_pair_step(BwdPair& p, float2 e, float4 q3,
     p.T = __fmul2_rn(p.T, oma);
   }
   const float2 wgt = __fmul2_rn(dLda, make_float2(live0 ? alpha.x : 0.f, live1 ? alpha.y : 0.f));
-  return make_float4(on0 ? wgt.x : 0.f, on1 ? wgt.y : 0.f, wE.x, wE.y);
+  const float2 wdy = __fmul2_rn(wgt, dy);
+  const float2 wdyy = __fmul2_rn(wdy, dy);
+  const float2 c0 = __fmul2_rn(p.g0, wE), c1 = __fmul2_rn(p.g1, wE), c2 = __fmul2_rn(p.g2, wE);
+  v[5] = wgt.x + wgt.y;
+  v[1] = wdy.x + wdy.y;
+  v[4] = wdyy.x + wdyy.y;
+  v[0] = dx.x * v[5];
+  v[2] = dx.x * v[0];
+  v[3] = dx.x * v[1];
+  v[6] = c0.x + c0.y;
+  v[7] = c1.x + c1.y;
+  v[8] = c2.x + c2.y;
 }
 
 template <int TW, int TH, int KIND, int CH, bool AHEAD>
@@ -835,7 +799,7 @@ __device__ __forceinline__ void backward_tile_pairs(const float4* __restrict__ r
                                                     const ViewParams* __restrict__ views,
                                                     const float* __restrict__ dl_dimage,
                                                     const float4* __restrict__ state, float4* __restrict__ grad2d,
-                                                    uint32_t tile, PairStageBuf<CH, true>& sb, ReplayWarp& rw) {
+                                                    uint32_t tile, PairStageBuf<CH>& sb) {
   using G = TileGeom<TW, TH, kBwdPix>;
   constexpr int B = G::kThreads;
   const TileView tv = tile_view(rp, views, (uint32_t)tile);
@@ -873,11 +837,7 @@ __device__ __forceinline__ void backward_tile_pairs(const float4* __restrict__ r
       if (g[k][0] == 0.f && g[k][1] == 0.f && g[k][2] == 0.f) last[k] = range.x;
     }
   }
-  const bool odd = replay_begin(rw, g[0], g[1], lane), odd_warp = __any_sync(kFull, odd);
-  const float bx = __shfl_sync(kFull, px[0], 0), by = __shfl_sync(kFull, py[0], 0);
-  ReplaySlot slot = {0.f, 0.f, 0u};
-  uint32_t slots = 0;
-  p.px = px[0];  // one column: px[1] == px[0]
+  p.px = make_float2(px[0], px[0]);  // one column: px[1] == px[0]
   p.py = make_float2(py[0], py[1]);
   p.last0 = last[0];
   p.last1 = last[1];
@@ -898,39 +858,45 @@ __device__ __forceinline__ void backward_tile_pairs(const float4* __restrict__ r
     __syncthreads();
     if (base < warp_last) {
       const int cnt = (int)(min(warp_last, min(base + (uint32_t)CH, range.y)) - base);
-      float2 e_next;
-      if constexpr (AHEAD) e_next = pair_log2_alpha(p, sb.r0[0], sb.q2[0]);
+      float2 dx_next, dy_next, e_next;
+      if constexpr (AHEAD) e_next = pair_log2_alpha(p, sb.q0[0], sb.q1[0], sb.q2[0], dx_next, dy_next);
       for (int j = 0; j < cnt; ++j) {
-        const float4 r0 = sb.r0[j];
-        float2 e;
+        float2 dx, dy, e;
         if constexpr (AHEAD) {  // the next entry's, while this one is differentiated
+          dx = dx_next;
+          dy = dy_next;
           e = e_next;
-          e_next = pair_log2_alpha(p, sb.r0[j + 1], sb.q2[j + 1]);
+          e_next = pair_log2_alpha(p, sb.q0[j + 1], sb.q1[j + 1], sb.q2[j + 1], dx_next, dy_next);
         } else {
-          e = pair_log2_alpha(p, r0, sb.q2[j]);
+          e = pair_log2_alpha(p, sb.q0[j], sb.q1[j], sb.q2[j], dx, dy);
         }
         const uint32_t pos = base + j;
         const bool on0 = pos < p.last0 && e.x >= rp.log2_alpha_min;
         const bool on1 = pos < p.last1 && e.y >= rp.log2_alpha_min;
-        if (__any_sync(kFull, on0 || on1)) {  // the step is exact for the pixels that are off
-          const float4 q3 = sb.q3[j];
-          const float4 w = bwd_pair_step<KIND>(p, e, q3, on0, on1, rp);
-          rw.w[slots * kSlotStride + lane] = w;
-          if ((uint32_t)(lane & (kSlots - 1)) == slots) slot = {r0.x, r0.y, __float_as_uint(q3.w)};
-          if (odd_warp && odd) {
-            float* dst = reinterpret_cast<float*>(grad2d + 3 * (size_t)__float_as_uint(q3.w));
-            if (on0) replay_odd_lane(dst, p.g0.x, p.g1.x, p.g2.x, w.z);
-            if (on1) replay_odd_lane(dst, p.g0.y, p.g1.y, p.g2.y, w.w);
-          }
-          if (++slots == kSlots) {
-            replay_flush(rw, slot, kSlots, bx, by, grad2d, lane);
-            slots = 0;
+        const bool on = on0 || on1;
+        const uint32_t mask = __ballot_sync(kFull, on);
+        if (mask) {  // warp-uniform: the step is exact for the lanes that are off
+          float v[9];
+          const float4 q4 = sb.q4[j];
+          bwd_pair_step<KIND>(p, e, dx, dy, sb.q3[j], q4, on0, on1, rp, v);
+          float4* dst = grad2d + 3 * (size_t)__float_as_uint(q4.z);
+          if (__popc(mask) <= kDirectLanes) {
+            if (on) {
+              atomicAdd(dst, make_float4(v[0], v[1], v[2], v[3]));
+              atomicAdd(dst + 1, make_float4(v[4], v[5], v[6], v[7]));
+              atomicAdd(reinterpret_cast<float*>(dst + 2), v[8]);
+            }
+          } else {
+            if (!on) {
+#pragma unroll
+              for (int k = 0; k < 9; ++k) v[k] = 0.f;
+            }
+            warp_reduce9_add(v, reinterpret_cast<float*>(dst), lane);
           }
         }
       }
     }
   }
-  if (slots) replay_flush(rw, slot, slots, bx, by, grad2d, lane);
 }
 
 template <int TW, int TH, int KIND, int CH>
@@ -939,7 +905,7 @@ __device__ __forceinline__ void backward_tile(const float4* __restrict__ rec, co
                                               const ViewParams* __restrict__ views,
                                               const float* __restrict__ dl_dimage, const float4* __restrict__ state,
                                               float4* __restrict__ grad2d, uint32_t tile, StageBuf<CH>& sb,
-                                              uint32_t* s_id, ReplayWarp& rw) {
+                                              uint32_t* s_id) {
   using G = TileGeom<TW, TH, kBwdPix>;
   constexpr int B = G::kThreads;
   static_assert(kBwdPix == 2, "the replay below is written for two pixels per thread");
@@ -991,11 +957,6 @@ __device__ __forceinline__ void backward_tile(const float4* __restrict__ rec, co
       if (q.g0 == 0.f && q.g1 == 0.f && q.g2 == 0.f) q.last = range.x;
     }
   }
-  const float ga[3] = {p[0].g0, p[0].g1, p[0].g2}, gb[3] = {p[1].g0, p[1].g1, p[1].g2};
-  const bool odd = replay_begin(rw, ga, gb, lane), odd_warp = __any_sync(kFull, odd);
-  const float bx = __shfl_sync(kFull, p[0].px, 0), by = __shfl_sync(kFull, p[0].py, 0);
-  ReplaySlot slot = {0.f, 0.f, 0u};
-  uint32_t slots = 0;
   // the warp walks entries up to the largest stop of its pixels
   const uint32_t warp_last = __reduce_max_sync(kFull, max(p[0].last, p[1].last));
   for (uint32_t base = range.x; base < range.y; base += CH) {
@@ -1008,41 +969,38 @@ __device__ __forceinline__ void backward_tile(const float4* __restrict__ rec, co
       for (int j = 0; j < cnt; ++j) {
         const uint32_t pos = base + j;
         const float4 r0 = sb.r0[j], r1 = sb.r1[j];
-        // both pixels of the thread lie in one column: dx and A' dx are shared
+        // both pixels of the thread lie in one column: dx and A' dx are shared, and the dx moments
+        // follow from the others (sum w dx = dx sum w, sum w dx^2 = dx^2 sum w, sum w dx dy = dx sum w dy)
         const float dx = __fsub_rn(p[0].px, r0.x), adx = __fmul_rn(r0.z, dx);
-        float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
-        const bool on0 = bwd_step<KIND>(p[0], dx, adx, r0, r1, sb.e2[j], pos, rp, w.x, w.z);
-        const bool on1 = bwd_step<KIND>(p[1], dx, adx, r0, r1, sb.e2[j], pos, rp, w.y, w.w);
-        if (__any_sync(kFull, on0 || on1)) {
-          rw.w[slots * kSlotStride + lane] = w;
-          if ((uint32_t)(lane & (kSlots - 1)) == slots) slot = {r0.x, r0.y, s_id[j]};
-          if (odd_warp && odd) {
-            float* dst = reinterpret_cast<float*>(grad2d + 3 * (size_t)s_id[j]);
-            if (on0) replay_odd_lane(dst, p[0].g0, p[0].g1, p[0].g2, w.z);
-            if (on1) replay_odd_lane(dst, p[1].g0, p[1].g1, p[1].g2, w.w);
-          }
-          if (++slots == kSlots) {
-            replay_flush(rw, slot, kSlots, bx, by, grad2d, lane);
-            slots = 0;
+        float v[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        bool on = bwd_step<KIND>(p[0], dx, adx, r0, r1, sb.e2[j], pos, rp, v);
+        on |= bwd_step<KIND>(p[1], dx, adx, r0, r1, sb.e2[j], pos, rp, v);
+        v[0] = dx * v[5];
+        v[2] = dx * v[0];
+        v[3] = dx * v[1];
+        const uint32_t mask = __ballot_sync(kFull, on);
+        if (mask) {
+          float4* dst = grad2d + 3 * (size_t)s_id[j];
+          // up to kDirectLanes lanes add their values with their own vector atomics (3 instructions) rather
+          // than through the warp reduction (about 70); a full warp hitting one splat reduces first, since
+          // 32 atomics on one address serialise
+          if (__popc(mask) <= kDirectLanes) {
+            if (on) {
+              atomicAdd(dst, make_float4(v[0], v[1], v[2], v[3]));
+              atomicAdd(dst + 1, make_float4(v[4], v[5], v[6], v[7]));
+              atomicAdd(reinterpret_cast<float*>(dst + 2), v[8]);
+            }
+          } else {
+            warp_reduce9_add(v, reinterpret_cast<float*>(dst), lane);
           }
         }
       }
     }
   }
-  if (slots) replay_flush(rw, slot, slots, bx, by, grad2d, lane);
 }
 
-// Shared memory of a replay CTA: the staged chunk, then each warp's gathered entries.
-template <int TW, int TH, int KIND, int CH>
-struct ReplayShared {
-  std::conditional_t<kPairForm<KIND, CH>, PairStageBuf<CH, true>, StageBuf<CH>> sb;
-  uint32_t id[kPairForm<KIND, CH> ? 4 : CH];  // the packed form carries the index in its q4
-  ReplayWarp warps[TW * TH / 64];
-};
-
-// 28 warps per SM: 72 registers, which the kernels just need (four bytes of spills in some).
 template <int TW, int TH, int KIND, int CH, Walk WALK>
-__global__ void __launch_bounds__(TW* TH / kBwdPix, 28 * 64 / (TW * TH)) composite_backward_kernel(const float4* __restrict__ rec,
+__global__ void __launch_bounds__(TW* TH / kBwdPix) composite_backward_kernel(const float4* __restrict__ rec,
                                                                         const uint32_t* __restrict__ ids,
                                                                         const uint2* __restrict__ ranges,
                                                                         RenderParams rp,
@@ -1053,14 +1011,14 @@ __global__ void __launch_bounds__(TW* TH / kBwdPix, 28 * 64 / (TW * TH)) composi
                                                                         const uint32_t* __restrict__ work,
                                                                         uint32_t* counter) {
   pdl_wait();
-  extern __shared__ __align__(16) unsigned char s_replay[];
-  ReplayShared<TW, TH, KIND, CH>& sh = *reinterpret_cast<ReplayShared<TW, TH, KIND, CH>*>(s_replay);
-  ReplayWarp& rw = sh.warps[threadIdx.x >> 5];
+  using Buf = std::conditional_t<kPairForm<KIND, CH>, PairStageBuf<CH>, StageBuf<CH>>;
+  __shared__ Buf sb;
+  __shared__ uint32_t s_id[kPairForm<KIND, CH> ? 1 : CH];  // the packed form carries the index in its q4
   auto one_tile = [&](uint32_t tile) {
     if constexpr (kPairForm<KIND, CH>)
-      backward_tile_pairs<TW, TH, KIND, CH, WALK == kAhead>(rec, ids, ranges, rp, views, dl_dimage, state, grad2d, tile, sh.sb, rw);
+      backward_tile_pairs<TW, TH, KIND, CH, WALK == kAhead>(rec, ids, ranges, rp, views, dl_dimage, state, grad2d, tile, sb);
     else
-      backward_tile<TW, TH, KIND, CH>(rec, ids, ranges, rp, views, dl_dimage, state, grad2d, tile, sh.sb, sh.id, rw);
+      backward_tile<TW, TH, KIND, CH>(rec, ids, ranges, rp, views, dl_dimage, state, grad2d, tile, sb, s_id);
   };
   if constexpr (WALK == kPersistent) {
     __shared__ uint32_t s_next;
@@ -1085,9 +1043,9 @@ struct Launch {
 
 // One CTA per tile, or one wave of persistent CTAs (SM count x resident CTAs per SM).
 template <typename Kernel>
-static unsigned grid_for(Kernel k, int threads, size_t shared, const Launch& L, uint32_t n_tiles) {
+static unsigned grid_for(Kernel k, int threads, const Launch& L, uint32_t n_tiles) {
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, shared) != cudaSuccess || per_sm < 1) per_sm = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
   return (unsigned)std::min<uint64_t>((uint64_t)per_sm * (uint64_t)L.num_sms, n_tiles);
 }
 
@@ -1108,7 +1066,7 @@ void forward_launch(const float4* rec, const uint32_t* ids, const uint2* ranges,
     k = composite_forward_kernel<TW, TH, KIND, CH, kPairFwd<TW, TH, KIND, CH> ? kAhead : kTiles>;
   } else if (L.counter) {
     k = composite_forward_kernel<TW, TH, KIND, CH, kPersistent>;
-    grid = grid_for(k, threads, 0, L, rp.n_tiles);
+    grid = grid_for(k, threads, L, rp.n_tiles);
   }
   launch_pdl(k, grid, threads, 0, s, rec, ids, ranges, rp, views, image, overdraw, state, L.work, L.counter);
 }
@@ -1119,20 +1077,14 @@ void backward_launch(const float4* rec, const uint32_t* ids, const uint2* ranges
                      cudaStream_t s) {
   constexpr int threads = TileGeom<TW, TH, kBwdPix>::kThreads;
   auto k = composite_backward_kernel<TW, TH, KIND, CH, kTiles>;
-  constexpr size_t shared = sizeof(ReplayShared<TW, TH, KIND, CH>);
   unsigned grid = rp.n_tiles;
   if (kPairForm<KIND, CH> && few_tiles<TW, TH>(L, rp.n_tiles)) {
     k = composite_backward_kernel<TW, TH, KIND, CH, kPairForm<KIND, CH> ? kAhead : kTiles>;
   } else if (L.counter) {
     k = composite_backward_kernel<TW, TH, KIND, CH, kPersistent>;
+    grid = grid_for(k, threads, L, rp.n_tiles);
   }
-  if (shared > 48 * 1024 &&
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared) != cudaSuccess)
-    return;  // the launch sequence's error check reports it
-  if (k == composite_backward_kernel<TW, TH, KIND, CH, kPersistent>) {
-    grid = grid_for(k, threads, shared, L, rp.n_tiles);
-  }
-  launch_pdl(k, grid, threads, shared, s, rec, ids, ranges, rp, views, dl, state, grad2d, L.work, L.counter);
+  launch_pdl(k, grid, threads, 0, s, rec, ids, ranges, rp, views, dl, state, grad2d, L.work, L.counter);
 }
 
 template <int TW, int TH, int KIND>
